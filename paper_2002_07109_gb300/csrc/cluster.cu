@@ -22,9 +22,9 @@
 // list within r + prune skin of some atom of I at the current positions,
 // so that the pair kernel reads a list close to the pairs it must evaluate
 // while the outer lists, with a larger skin, are rebuilt rarely.
-// Pair kernel: one warp per work item (cluster I, chunk of BOUNCE_CL_EPW
-// pruned entries); lane = one list atom j, the 8 atoms
-// of cluster I in turn from shared memory.  Every unordered pair inside the
+// Pair kernel: one warp per work item (cluster I, a chunk of its pruned
+// entries); lane = one list atom j, the 8 atoms
+// of cluster I two at a time from shared memory.  Every unordered pair inside the
 // cutoff is evaluated once (Newton's third law): the j-side sum of a lane is
 // added once per item, the i-side sums are reduced over the warp at the end
 // of the item, both into int64 fixed-point accumulators (2^-32 kcal/mol/A)
@@ -35,13 +35,17 @@
 #include <cstdint>
 
 #include "common.cuh"
+#include "pairs.cuh"
 
 namespace {
 
-// resident CTAs per SM the pair kernel is compiled for (register budget)
-#ifndef CL_PAIRS_MIN_CTAS
-#define CL_PAIRS_MIN_CTAS 3
+// Threads per CTA of the pair kernel and the resident CTAs per SM it is
+// compiled for: 128 registers a thread, 16 warps per SM.  96 registers (20
+// warps) spill and were slower, 121 against 105 us on the 98,304-atom box.
+#ifndef X_CTAS
+#define X_CTAS 4
 #endif
+constexpr int PAIRS_NT = 128, PAIRS_CTAS = X_CTAS;
 
 constexpr int CL = BOUNCE_CL;
 constexpr int EPW = BOUNCE_CL_EPW;
@@ -479,7 +483,7 @@ __global__ void __launch_bounds__(256) k_cl_prune(DevSys s, Params p, int step_o
                 const int nch = (m + EPW - 1) / EPW;
                 const int b = nch ? atomicAdd(&c.pnitems[2 + L], nch) : 0;
                 for (int k = 0; k < nch; ++k)
-                    if (b + k < c.capitems) c.pitems[L][b + k] = make_int2(I, k * EPW);
+                    if (b + k < c.capitems) c.pitems[L][b + k] = make_int4(I, k * EPW, min((k + 1) * EPW, m), 0);
             }
         }
     }
@@ -493,171 +497,169 @@ __global__ void __launch_bounds__(256) k_cl_prune(DevSys s, Params p, int step_o
     if (threadIdx.x == 0) *c.prune = 0;
 }
 
-__device__ __forceinline__ void fix_add(unsigned long long* a, float v) {
-    if (v != 0.f) atomicAdd(a, fix_round<32>(v));
-}
-
-// Exact FP64 cutoff test of one pair near r_c, out of line (rare).
-__device__ __noinline__ bool cl_exact_inside(const DevSys& s, const Params& p, int cur, int a, int b) {
-    return exact_r2(s, p, cur, a, b) < p.rc2_d;
-}
-
-
 // The pairs of one list entry (atom slot sj, split position hj/lj in the
-// image of the entry) whose FP32 r^2 fell within the rounding band of r_c^2
-// (bits of `near`): each takes the exact FP64 cutoff test; a pair inside
-// adds its i side straight to the accumulator of its slot (rare) and its j
-// side to the lane's sums.
+// image of the entry) whose FP32 r^2 falls within the rounding band of r_c^2:
+// each takes the exact FP64 cutoff test; a pair inside adds its i side
+// straight to the accumulator of its slot; the j side gj with the pairs added
+// and their number are returned (by value: the caller's sums stay in
+// registers).  Rare (the band is 2e-5 of r_c^2 wide), so kept out of the
+// unrolled code.
 template <int PART>
-__device__ __forceinline__ void near_pairs(const DevSys& s, const Params& p, int cur, int I, int sj, float4 hj, float4 lj,
-                                        uint32_t near, const float4* s_hi, const float4* s_lo, const float* s_c12,
-                                        const float* s_c6, float& gjx, float& gjy, float& gjz, int& npair) {
+__device__ __noinline__ float4 near_pairs(const DevSys& s, const Params& p, int cur, int I, int sj, float4 hj, float4 lj,
+                                          int mj, int above, float3 gj) {
     const DevClu& c = s.cl;
+    int npair = 0;
     const size_t ns = (size_t)c.ncol * c.maxcl * CL;
-    for (; near; near &= near - 1u) {
-        const int a = __ffs(near) - 1;
-        if (!(exact_r2(s, p, cur, c.cl_atom[I * CL + a], c.cl_atom[sj]) < p.rc2_d)) continue;
-        const float4 hi = s_hi[a], lo = s_lo[a];
+    for (int a = 0; a < min(CL, above); ++a) {
+        const int si = I * CL + a;
+        if (c.smol[si] < 0 || c.smol[si] == mj) continue;
+        const float4 hi = c.sphi[cur][si], lo = c.splo[cur][si];
         const float3 d = pair_disp(p, hi, lo, hj, lj);
         const float r2 = d.x * d.x + d.y * d.y + d.z * d.z;
+        if (!(r2 >= p.rc2_lo && r2 <= p.rc2_hi)) continue;
+        if (!(exact_r2(s, p, cur, c.cl_atom[si], c.cl_atom[sj]) < p.rc2_d)) continue;
         const int tp = type_of(lo) * BOUNCE_MAXT + type_of(lj);
-        const float w = pairsum_w<PART>(p, r2, p.kcoul * hi.w * hj.w, s_c12[tp], s_c6[tp]);
-        fix_add(c.acc + (size_t)I * CL + a, w * d.x);
-        fix_add(c.acc + ns + (size_t)I * CL + a, w * d.y);
-        fix_add(c.acc + 2 * ns + (size_t)I * CL + a, w * d.z);
-        gjx = fmaf(-w, d.x, gjx);
-        gjy = fmaf(-w, d.y, gjy);
-        gjz = fmaf(-w, d.z, gjz);
+        const float w = pairsum_w<PART>(p, r2, p.kcoul * hi.w * hj.w, p.c12[tp], p.c6[tp]);
+        fix_add(c.acc + si, w * d.x);
+        fix_add(c.acc + ns + si, w * d.y);
+        fix_add(c.acc + 2 * ns + si, w * d.z);
+        gj.x = fmaf(-w, d.x, gj.x);
+        gj.y = fmaf(-w, d.y, gj.y);
+        gj.z = fmaf(-w, d.z, gj.z);
         ++npair;
     }
-}
-
-// The 8 pairs of one list entry j (split position hj/lj in the entry's
-// image, molecule mj, type tj, slot sj) with the atoms of cluster I (shared
-// memory): i sides into gi, the j side into gj, in-cutoff pairs counted,
-// pairs within the rounding band of r_c flagged in `near` for the exact
-// test.  PER: minimum image per pair (clusters near half a box edge).
-template <int PART, bool PER>
-__device__ __forceinline__ void entry_pairs(const Params& p, const float4* shi, const float4* slo, const int* smol,
-                                            const float* c12t, const float* c6t, float4 hj, float4 lj, int mj, int tj,
-                                            int sj, int I, float (&gi)[CL][3], float& gjx, float& gjy, float& gjz,
-                                            uint32_t& near, int& npair) {
-#pragma unroll
-    for (int a = 0; a < CL; ++a) {
-        const float4 hi = shi[a], lo = slo[a];
-        const int mi = smol[a];
-        float3 d;
-        if (PER) {
-            d = pair_disp(p, hi, lo, hj, lj);
-        } else {
-            d.x = (hi.x - hj.x) + (lo.x - lj.x);
-            d.y = (hi.y - hj.y) + (lo.y - lj.y);
-            d.z = (hi.z - hj.z) + (lo.z - lj.z);
-        }
-        const float r2 = d.x * d.x + d.y * d.y + d.z * d.z;
-        const bool ok = mi >= 0 && mi != mj && sj > I * CL + a;
-        const bool in = ok && r2 < p.rc2_lo;
-        near |= (ok && r2 >= p.rc2_lo && r2 <= p.rc2_hi) ? 1u << a : 0u;
-        const int tp = type_of(lo) * BOUNCE_MAXT + tj;
-        const float w0 = pairsum_w<PART>(p, in ? r2 : 1.f, p.kcoul * hi.w * hj.w, c12t[tp], c6t[tp]);
-        const float wv = in ? w0 : 0.f;
-        npair += in ? 1 : 0;
-        gi[a][0] = fmaf(wv, d.x, gi[a][0]);
-        gi[a][1] = fmaf(wv, d.y, gi[a][1]);
-        gi[a][2] = fmaf(wv, d.z, gi[a][2]);
-        gjx = fmaf(-wv, d.x, gjx);
-        gjy = fmaf(-wv, d.y, gjy);
-        gjz = fmaf(-wv, d.z, gjz);
-    }
+    return make_float4(gj.x, gj.y, gj.z, __int_as_float(npair));
 }
 
 // Pair sums over the work items of list `L`.  PART 3: the F_0 share
 // (1 - chi) W'_sw + W'_fixed; PART 5: the full W'.  A warp takes an item of
 // cluster I: lanes hold one list atom j each, the 8 atoms of I are read from
-// shared memory in turn; the j side of every pair is summed in the lane's
-// registers and added once per item, the i side is kept per lane for the 8
-// atoms and reduced over the warp at the end of the item.
-template <int PART>
-__global__ void __launch_bounds__(256, CL_PAIRS_MIN_CTAS) k_cl_pairs(DevSys s, Params p, int step_off, int L) {
+// shared memory two at a time (pairs.cuh); the j side of every pair is summed
+// in the lane's registers and added once per entry, the i side is kept per
+// lane for the 8 atoms and reduced over the warp at the end of the item.
+//
+// Bound by instruction issue and the latency that 16 warps per SM leave
+// uncovered.  98,304-atom water box, per launch: 109 us for the F_0 share and
+// 96 us for the full sums, against 165 and 145 with one pair per instruction;
+// 12,288-atom droplet (r_c 12 A) 35 against 55 us.  What it took besides the
+// packed arithmetic: the j atoms of the next pass are gathered into registers
+// while this one is evaluated, across items too; reductions to global memory
+// instead of generic atomics, and near_pairs by value instead of through the
+// stack (together 12 us of the box's 117).
+template <int PART, bool EW, bool CJ>
+__global__ void __launch_bounds__(PAIRS_NT, PAIRS_CTAS) k_cl_pairs(const __grid_constant__ DevSys s,
+                                                                   const __grid_constant__ Params p,
+                                                                   const __grid_constant__ PairConsts k, int step_off,
+                                                                   int L) {
     chain_enter();
-    __shared__ float4 s_hi[8][CL], s_lo[8][CL];
-    __shared__ int s_mol[8][CL];
-    __shared__ float s_c12[BOUNCE_MAXT * BOUNCE_MAXT], s_c6[BOUNCE_MAXT * BOUNCE_MAXT];
-    if (threadIdx.x < BOUNCE_MAXT * BOUNCE_MAXT) {
-        s_c12[threadIdx.x] = p.c12[threadIdx.x];
-        s_c6[threadIdx.x] = p.c6[threadIdx.x];
-    }
-    __syncthreads();
+    __shared__ IGroup s_g[PAIRS_NT / 32];
     const DevClu& c = s.cl;
-    const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
+    IGroup& g = s_g[threadIdx.x >> 5];
     const int cur = (int)((*s.step_base + step_off) & 1);
     const int capj = c.capj[L];
-    const int* lst = c.plst[L];
-    const int* lcnt = c.pcnt[L];
     const int nit = c.pnitems[L];
     const size_t ns = (size_t)c.ncol * c.maxcl * CL;
     const float4* sphi = c.sphi[cur];
     const float4* splo = c.splo[cur];
+    const int* plst = c.plst[L];
+    auto entry = [&](int4 it, int e) -> int {  // list entry e of item it (0 beyond its end)
+        return e < it.z ? __ldg(plst + (size_t)it.x * capj + e) : 0;
+    };
+    float4 nh, nl;  // j atom of the next pass
+    int nm;
+    auto gather = [&](int ent) {
+        nh = sphi[ent & 0x07FFFFFF];
+        nl = splo[ent & 0x07FFFFFF];
+        nm = c.smol[ent & 0x07FFFFFF];
+    };
     int npair = 0;
     // items are fetched from a counter, so that no warp idles while its
     // CTA's other warps still work (the items differ in length)
-    for (;;) {
-        int it = 0;
-        if (lane == 0) it = atomicAdd(&c.pnitems[4 + L], 1);
-        it = __shfl_sync(0xffffffffu, it, 0);
-        if (it >= nit) break;
-        const int2 w = c.pitems[L][it];
-        const int I = w.x, e1 = min(w.y + EPW, lcnt[I]);
-        __syncwarp();
-        if (lane < CL) {
-            s_hi[wl][lane] = sphi[I * CL + lane];
-            s_lo[wl][lane] = splo[I * CL + lane];
-            s_mol[wl][lane] = c.smol[I * CL + lane];
-        }
-        __syncwarp();
-        float gi[CL][3];
+    int nx = 0;
+    if (lane == 0) nx = atomicAdd(&c.pnitems[4 + L], 1);
+    nx = __shfl_sync(0xffffffffu, nx, 0);
+    if (nx < nit) {
+        int4 w = c.pitems[L][nx];  // (I, first entry, end, -)
+        int ent = entry(w, w.y + lane), ent1 = entry(w, w.y + 32 + lane);
+        gather(ent);
+        for (;;) {
+            const int I = w.x;
+            if (lane == 0) nx = atomicAdd(&c.pnitems[4 + L], 1);
+            // the next item: its number was asked for just now, its record is
+            // read after this item's first pass, its first entries after the second
+            int4 wn = make_int4(0, 0, 0, 0);
+            int stage = 0, nent = 0;
+            auto advance = [&]() {
+                if (stage == 0) {
+                    nx = __shfl_sync(0xffffffffu, nx, 0);
+                    if (nx < nit) wn = c.pitems[L][nx];
+                } else if (stage == 1) {
+                    nent = entry(wn, wn.y + lane);
+                }
+                ++stage;
+            };
+            __syncwarp();
+            if (lane < CL) igroup_set(g, p, lane, sphi[I * CL + lane], splo[I * CL + lane], c.smol[I * CL + lane]);
+            __syncwarp();
+            float2 gi[4][3];
 #pragma unroll
-        for (int a = 0; a < CL; ++a) gi[a][0] = gi[a][1] = gi[a][2] = 0.f;
-        for (int e = w.y + lane; e < e1; e += 32) {
-            const int ent = __ldg(lst + (size_t)I * capj + e);
-            const int sj = ent & 0x07FFFFFF, code = (int)((uint32_t)ent >> 27);
-            float4 hj = sphi[sj], lj = splo[sj];
-            const int mj = c.smol[sj];
-            const int tj = type_of(lj);
-            if (code != NO_SHIFT && code != PER_PAIR) {
-                const float kx = (float)(code / 9 - 1), ky = (float)((code / 3) % 3 - 1), kz = (float)(code % 3 - 1);
-                shift_split(hj.x, lj.x, kx * p.Lhi[0], kx * p.Llo[0]);
-                shift_split(hj.y, lj.y, ky * p.Lhi[1], ky * p.Llo[1]);
-                shift_split(hj.z, lj.z, kz * p.Lhi[2], kz * p.Llo[2]);
+            for (int a = 0; a < 4; ++a) gi[a][0] = gi[a][1] = gi[a][2] = make_float2(0.f, 0.f);
+            for (int e0 = w.y; e0 < w.z; e0 += 32) {
+                const bool valid = e0 + lane < w.z;  // (an entry's image code fills its top bits)
+                const int sj = ent & 0x07FFFFFF;
+                const int code = valid ? (int)((uint32_t)ent >> 27) : NO_SHIFT;
+                JAtom j;
+                j.h = nh;
+                j.l = nl;
+                j.mol = nm;
+                // the next pass's atoms, of this item or the next
+                if (e0 + 32 < w.z) {
+                    ent = ent1;
+                    gather(ent);
+                    ent1 = entry(w, e0 + 64 + lane);
+                } else {
+                    while (stage < 2) advance();
+                    ent = nent;
+                    gather(ent);
+                    ent1 = entry(wn, wn.y + 32 + lane);
+                }
+                j.type = type_of(j.l);
+                // pairs within I: the lower slot is i (every other j lies in a later cluster)
+                j.above = valid ? sj - I * CL : 0;
+                if (code != NO_SHIFT && code != PER_PAIR) {
+                    const float kx = (float)(code / 9 - 1), ky = (float)((code / 3) % 3 - 1), kz = (float)(code % 3 - 1);
+                    shift_split(j.h.x, j.l.x, kx * p.Lhi[0], kx * p.Llo[0]);
+                    shift_split(j.h.y, j.l.y, ky * p.Lhi[1], ky * p.Llo[1]);
+                    shift_split(j.h.z, j.l.z, kz * p.Lhi[2], kz * p.Llo[2]);
+                }
+                if (!valid) j.h.x = PAIR_FAR;
+                float3 gs = make_float3(0.f, 0.f, 0.f);
+                float near = INFINITY;
+                // entries of the own cluster (index rule) or near half a box edge
+                // (minimum image per pair) take their warp through a copy of the
+                // loop with both (the same sums for the other entries)
+                if (__any_sync(0xffffffffu, code == PER_PAIR || (valid && j.above < CL)))
+                    group_pairs<PART, EW, CJ, true>(k, g, j, gi, gs, near, npair);
+                else
+                    group_pairs<PART, EW, CJ, false>(k, g, j, gi, gs, near, npair);
+                if (near <= k.band) {
+                    const float4 o = near_pairs<PART>(s, p, cur, I, sj, j.h, j.l, j.mol, j.above, gs);
+                    gs = make_float3(o.x, o.y, o.z);
+                    npair += __float_as_int(o.w);
+                }
+                fix_add(c.acc + sj, gs.x);
+                fix_add(c.acc + ns + sj, gs.y);
+                fix_add(c.acc + 2 * ns + sj, gs.z);
+                if (stage < 2) advance();
             }
-            float gjx = 0.f, gjy = 0.f, gjz = 0.f;
-            uint32_t near = 0u;  // pairs within the FP32 rounding band of r_c
-            // the rare per-pair minimum image takes its own copy of the loop,
-            // so that the common one carries no minimum-image arithmetic
-            if (code == PER_PAIR)
-                entry_pairs<PART, true>(p, s_hi[wl], s_lo[wl], s_mol[wl], s_c12, s_c6, hj, lj, mj, tj, sj, I, gi, gjx,
-                                        gjy, gjz, near, npair);
-            else
-                entry_pairs<PART, false>(p, s_hi[wl], s_lo[wl], s_mol[wl], s_c12, s_c6, hj, lj, mj, tj, sj, I, gi, gjx,
-                                         gjy, gjz, near, npair);
-            if (near) near_pairs<PART>(s, p, cur, I, sj, hj, lj, near, s_hi[wl], s_lo[wl], s_c12, s_c6, gjx, gjy, gjz,
-                                       npair);
-            fix_add(c.acc + sj, gjx);
-            fix_add(c.acc + ns + sj, gjy);
-            fix_add(c.acc + 2 * ns + sj, gjz);
+            // i side: lane 4 b + d adds component d of atom igroup_atom(b)
+            const float mine = igroup_reduce(gi);
+            const int a = igroup_atom(lane >> 2), d = lane & 3;
+            if (d < 3) fix_add(c.acc + (size_t)d * ns + I * CL + a, mine);
+            if (nx >= nit) break;
+            w = wn;
         }
-        // i side: each of the 24 sums over the warp; lane 3 a + d adds component d of atom a
-        float mine = 0.f;
-#pragma unroll
-        for (int a = 0; a < CL; ++a)
-#pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                float v = gi[a][d];
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                if (lane == 3 * a + d) mine = v;
-            }
-        if (lane < 3 * CL && s_mol[wl][lane / 3] >= 0) fix_add(c.acc + (size_t)(lane % 3) * ns + I * CL + lane / 3, mine);
     }
     npair = warp_sum_i(npair);
     if (lane == 0 && npair) atomicAdd(&s.cnt[PART == 3 ? CNT_SHORT_PAIRS : CNT_FULL_PAIRS], (unsigned long long)npair);
@@ -693,29 +695,49 @@ void launch_cluster_rebuild(const DevSys& s, const Params& p, int step_off, bool
     launch_chained(k_cl_prune, std::min((ncl + 7) / 8, 152 * 8), 256, 0, st, s, p, step_off, f);
 }
 
-// CTAs of the pair kernel that fit on the GPU at once (the warps fetch their
+// CTAs of a pair kernel that fit on the GPU at once (the warps fetch their
 // work items, so one resident wave covers any number of items)
-template <int PART>
-static int cl_pairs_grid() {
-    static int blocks = 0;
+template <typename K>
+static int resident_ctas(K kernel, int& blocks) {
     if (!blocks) {
         int dev = 0, sms = 0, per = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_cl_pairs<PART>, 256, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, PAIRS_NT, 0);
         blocks = std::max(1, sms * std::max(per, 1));
     }
     return blocks;
 }
 
+template <int PART, bool EW, bool CJ>
+static int cl_pairs_grid() {
+    static int blocks = 0;
+    return resident_ctas(k_cl_pairs<PART, EW, CJ>, blocks);
+}
+
 void prepare_cluster_pairs() {
-    cl_pairs_grid<3>();
-    cl_pairs_grid<5>();
+    cl_pairs_grid<5, true, true>();
+    cl_pairs_grid<5, false, true>();
+    cl_pairs_grid<3, true, true>();
+    cl_pairs_grid<3, true, false>();
+    cl_pairs_grid<3, false, true>();
+    cl_pairs_grid<3, false, false>();
+}
+
+template <int PART, bool CJ>
+static void launch_cl_pairs(const DevSys& s, const Params& p, int step_off, int list, cudaStream_t st) {
+    const PairConsts k = make_pair_consts(p);
+    if (p.ebeta > 0.f)
+        launch_chained(k_cl_pairs<PART, true, CJ>, cl_pairs_grid<PART, true, CJ>(), PAIRS_NT, 0, st, s, p, k, step_off, list);
+    else
+        launch_chained(k_cl_pairs<PART, false, CJ>, cl_pairs_grid<PART, false, CJ>(), PAIRS_NT, 0, st, s, p, k, step_off,
+                       list);
 }
 
 void launch_cluster_pairs(const DevSys& s, const Params& p, int step_off, int part, int list, cudaStream_t st) {
-    if (part == 3) launch_chained(k_cl_pairs<3>, cl_pairs_grid<3>(), 256, 0, st, s, p, step_off, list);
-    else launch_chained(k_cl_pairs<5>, cl_pairs_grid<5>(), 256, 0, st, s, p, step_off, list);
+    if (part != 3) launch_cl_pairs<5, true>(s, p, step_off, list, st);
+    else if (p.coul_jump) launch_cl_pairs<3, true>(s, p, step_off, list, st);
+    else launch_cl_pairs<3, false>(s, p, step_off, list, st);
 }
 
 void launch_cluster_collect(const DevSys& s, double* out, cudaStream_t st) {

@@ -34,10 +34,8 @@ constexpr double ACCEL_D = 4.184e-4;
 // sums both sides of every pair once (Newton's third law) into int64
 // fixed-point accumulators, one per slot and component.
 #define BOUNCE_CL 8
-#ifndef BOUNCE_CL_EPW
 #define BOUNCE_CL_EPW 512          // list entries per work item of the pair kernel (one item per
                                    // cluster on the water box: fewer i-side reductions)
-#endif
 #define BOUNCE_CL_MAXCOL 1024      // atoms per column (one CTA sorts a column in shared memory)
 constexpr double CL_FIX = 4294967296.0;        // fixed-point scale 2^32 of the accumulators
 constexpr double CL_UNFIX = 2.3283064365386963e-10;  // 2^-32
@@ -82,7 +80,7 @@ struct DevClu {
     // I at the last prune, valid while no atom moved half the prune skin
     int* plst[2];            // [ncl * capj] same layout as lst
     int* pcnt[2];            // [ncl]
-    int2* pitems[2];         // (I, first entry) of each work item of the pruned lists, in allocation order
+    int4* pitems[2];         // (I, first entry, end, -) of each work item of the pruned lists, in allocation order
     int* pnitems;            // [2] work items, [2..3] their allocation counters, [4..5] the
                              //     pair kernel's fetch counters (zero between launches)
     int capitems;            // work items per list
@@ -537,6 +535,15 @@ __device__ __forceinline__ unsigned long long fix_round(float v) {
     constexpr float scale = (float)(1ull << S);
     constexpr float vmax = (float)(1ull << (63 - S));
     return (unsigned long long)__float2ll_rn(fminf(fmaxf(v, -vmax), vmax) * scale);
+}
+
+// a += v in fixed point.  The address is known to be global memory here, but
+// not to the compiler (the pointers arrive inside a struct), which would take
+// the generic atomic; a reduction that returns nothing is asked for instead.
+__device__ __forceinline__ void fix_add(unsigned long long* a, float v) {
+    if (v != 0.f)
+        asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(__cvta_generic_to_global(a)), "l"(fix_round<32>(v))
+                     : "memory");
 }
 
 __device__ __forceinline__ float warp_sum_f(float x) {
