@@ -41,11 +41,9 @@ namespace {
 
 // Threads per CTA of the pair kernel and the resident CTAs per SM it is
 // compiled for: 128 registers a thread, 16 warps per SM.  96 registers (20
-// warps) spill and were slower, 121 against 105 us on the 98,304-atom box.
-#ifndef X_CTAS
-#define X_CTAS 4
-#endif
-constexpr int PAIRS_NT = 128, PAIRS_CTAS = X_CTAS;
+// warps) spill: 123 against 109 us on the 98,304-atom box; 168 registers (12
+// warps): 113 us.
+constexpr int PAIRS_NT = 128, PAIRS_CTAS = 4;
 
 constexpr int CL = BOUNCE_CL;
 constexpr int EPW = BOUNCE_CL_EPW;

@@ -98,6 +98,7 @@ struct DevTile {
     int nitems;
     int blocks;              // resident grid of the tile kernel
     int tj;                  // atoms per j-block
+    int pairs;               // items carry a second i-tile (k_tile_pairs; else k_tile_pairs1)
     const int4* items;
     unsigned long long* acc; // [3 n] (x, y, z blocks)
 };

@@ -38,6 +38,31 @@ def test_small_boxes(side, r_cut, vdw):
                                             max_neighbors=1024, jump_coulomb=not vdw))
 
 
+def test_paired_tiles_equal_single_tiles():
+    """A batch large enough that two i-tiles share an item gives, bit for bit,
+    the pair sums of each droplet alone (one tile an item): tile and block
+    remainders of 1 to 31 atoms, replicas of one tile, of one block, of an odd
+    number of blocks."""
+    from paper_2002_07109_gb300.water import concat_systems
+    sizes = [1, 10, 11, 21, 22, 43, 64, 85, 107] * 20
+    cat, off = concat_systems([water_droplet_molecules(m, seed=m) for m in sizes], spacing=0.0)
+    cfg = dict(DROP, jump_coulomb=False, max_neighbors=400)
+    ctx = bounce.from_system(cat, seed=1, **cfg)
+    ctx.set_replicas(off, np.arange(len(sizes), dtype=np.uint64))
+    ctx.set_state(cat.q, cat.v)
+    both = [ctx.gradient(code) for code in (bounce.GRAD_FULL, bounce.GRAD_SHORT)]
+    ctx.close()
+    for r, m in enumerate(sizes[:9]):
+        s = water_droplet_molecules(m, seed=m)
+        one = bounce.from_system(s, seed=1, **cfg)
+        one.set_state(s.q, s.v)
+        for g, code in zip(both, (bounce.GRAD_FULL, bounce.GRAD_SHORT)):
+            ref = one.gradient(code)
+            for k in range(r, len(sizes), 9):
+                assert np.array_equal(g[off[k]:off[k + 1]], ref), (m, k, code)
+        one.close()
+
+
 def _check(s, cfg):
     q = s.q + np.random.default_rng(7).normal(scale=0.05, size=s.q.shape) + 1.3   # some atoms outside the box
     ctx = bounce.from_system(s, seed=3, **cfg)
