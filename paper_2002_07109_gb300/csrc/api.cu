@@ -359,13 +359,16 @@ int setup_pme(bounce_ctx* c) {
     float* dbc;
     int *doff, *didx;
     int r;
+    m.row = (m.K[2] + PME_PAD + 3) & ~3;
     if ((r = dalloc(c, &m.qgrid, N)) || (r = dalloc(c, &m.cgrid, N)) || (r = dalloc(c, &dbc, N)) ||
-        (r = dalloc(c, &m.grad, 3 * (size_t)c->n)) || (r = dalloc(c, &m.eexcl, c->n)) || (r = dalloc(c, &m.eterm, 256)) ||
+        (r = dalloc(c, &m.rgrid, (size_t)m.K[0] * m.K[1] * m.row + 16)) ||  // (the gather's last read may pass the end)
+        (r = dalloc(c, &m.grad, 3 * (size_t)c->n)) || (r = dalloc(c, &m.frac, c->n)) || (r = dalloc(c, &m.eexcl, c->n)) || (r = dalloc(c, &m.eterm, 256)) ||
         (r = dalloc(c, &doff, c->n + 1)) || (r = dalloc(c, &didx, std::max<size_t>(idx.size(), 1))))
         return r;
     CU(cudaMemcpy(dbc, bc.data(), N * sizeof(float), cudaMemcpyHostToDevice));
     CU(cudaMemcpy(doff, off.data(), off.size() * sizeof(int), cudaMemcpyHostToDevice));
     if (!idx.empty()) CU(cudaMemcpy(didx, idx.data(), idx.size() * sizeof(int), cudaMemcpyHostToDevice));
+    prepare_pme();
     m.bc = dbc;
     m.ex_off = doff;
     m.ex_idx = didx;
@@ -1637,7 +1640,7 @@ int64_t bounce_run_launch_count(const bounce_ctx* c, int64_t n, int32_t integ) {
     const int64_t per_boundary = (clu ? 5 : 0) + ((clu && integ == BOUNCE_BAOAB) ? 0 : (c->ds.rep_of ? 1 : 3)) + 1;
     const bool ext = integ >= BOUNCE_BOUNCE_RESPA_EXT;
     const bool short_f0 = !clu && integ != BOUNCE_BAOAB && c->pp.rshort2 < INFINITY;
-    const int64_t pme_launches = 10; // spread, load, 3 + 3 transforms, convolve, gather
+    const int64_t pme_launches = c->has_pme ? pme_launch_count(c->pme) : 0;
     int64_t total = 2;               // step-counter updates after the head and the bodies
     for (int64_t k = 0; k <= n; ++k) {
         bool pme;

@@ -170,6 +170,7 @@ struct DevSys {
     int lite;                // thread-per-atom step kernel (rare jump proposals)
 };
 
+constexpr int PME_PAD = 8;
 // Smooth particle-mesh Ewald state (periodic boxes with a reciprocal part).
 struct DevPme {
     int K[3];
@@ -179,7 +180,10 @@ struct DevPme {
     float beta, two_b_sqrtpi;
     unsigned long long* qgrid;   // int64 fixed-point charge grid (2^40 scale)
     float2* cgrid;               // complex work grid
+    float* rgrid;                // real potential: rows of `row` floats, point z at PME_PAD + z, the PME_PAD floats
+    int row;                     //     before it the points below 0 (periodic); a multiple of 4
     const float* bc;             // influence function B(m) C(m)
+    float4* frac;                // [n] grid fractions of each atom, w: its grid point, 10 bits an axis (spread -> gather)
     double* grad;                // [3 n] SoA gradient of E_recip + E_excl
     double* eexcl;               // [n] exclusion energy per atom (pairs j > i)
     double* eterm;               // [256] energy partials of the convolution
@@ -538,13 +542,29 @@ __device__ __forceinline__ unsigned long long fix_round(float v) {
     return (unsigned long long)__float2ll_rn(fminf(fmaxf(v, -vmax), vmax) * scale);
 }
 
-// a += v in fixed point.  The address is known to be global memory here, but
-// not to the compiler (the pointers arrive inside a struct), which would take
-// the generic atomic; a reduction that returns nothing is asked for instead.
+// fix_round without the int64 conversion (which runs on the FP64 pipe, one
+// warp instruction per ~16 SM cycles): v 2^S = A 2^20 + B 2^20 with A =
+// rint(v 2^(S-20)) and |B| <= 1/2 exact, both rounded by adding 1.5 2^23.
+// A 2^20 is even, so the two roundings are the one of the whole, ties
+// included.  For |v| <= 2^(42-S); the conversion beyond.
+template <int S>
+__device__ __forceinline__ unsigned long long fix_round_int(float v) {
+    constexpr float magic = 12582912.f, sa = (float)(1ull << (S - 20)), sb = 1048576.f;
+    if (!(fabsf(v) <= (float)(1ull << (42 - S)))) return fix_round<S>(v);
+    const float t = __fmul_rn(v, sa), a = __fadd_rn(t, magic);
+    const float b = __fmaf_rn(__fsub_rn(t, __fsub_rn(a, magic)), sb, magic);
+    const int ai = __float_as_int(a) - __float_as_int(magic), bi = __float_as_int(b) - __float_as_int(magic);
+    return (unsigned long long)((long long)ai * 1048576ll + (long long)bi);
+}
+
+// *a += v.  The address is known to be global memory here, but not to the
+// compiler (the pointers arrive inside a struct), which would take the
+// generic atomic; a reduction that returns nothing is asked for instead.
+__device__ __forceinline__ void red_add(unsigned long long* a, unsigned long long v) {
+    asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(__cvta_generic_to_global(a)), "l"(v) : "memory");
+}
 __device__ __forceinline__ void fix_add(unsigned long long* a, float v) {
-    if (v != 0.f)
-        asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(__cvta_generic_to_global(a)), "l"(fix_round<32>(v))
-                     : "memory");
+    if (v != 0.f) red_add(a, fix_round<32>(v));
 }
 
 __device__ __forceinline__ float warp_sum_f(float x) {
@@ -641,6 +661,9 @@ void launch_step_kernel(const DevSys& s, const Params& p, int integrator, int va
                         double hout, int pre, cudaStream_t st);
 // energy: also the FP64 energy partials of the convolution (bounce_get_energies)
 void launch_pme(const DevSys& s, const Params& p, const DevPme& m, int step_off, cudaStream_t st, bool energy = false);
+int pme_launch_count(const DevPme& m);  // launches of one evaluation without the energy
+// sets the shared-memory limits of the SPME kernels (outside any graph capture)
+void prepare_pme();
 void launch_pme_energy(const DevPme& m, int n, double* out, cudaStream_t st);
 void launch_gradient(const DevSys& s, const Params& p, int part, int cur, double* out, cudaStream_t st);
 void launch_jump_half(const DevSys& s, const Params& p, int cur, long long step, int stream_id, int* M, int* nacc,

@@ -76,7 +76,7 @@ __device__ __forceinline__ void tile_stage(const PairConsts& k, const float4* sh
 
 __device__ __forceinline__ void fix_add2(unsigned long long* a, float v, float w) {
     const unsigned long long f = fix_round<32>(v) + fix_round<32>(w);
-    if (f) asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(__cvta_generic_to_global(a)), "l"(f) : "memory");
+    if (f) red_add(a, f);
 }
 
 // Bound by instruction issue (the six shuffles and the staged loads of a
