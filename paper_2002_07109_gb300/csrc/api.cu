@@ -27,6 +27,7 @@ void launch_msd(const DevSys& s, const double* rx, const double* ry, const doubl
 namespace {
 
 constexpr int CHUNK = 32;  // steps per captured graph
+constexpr int H_OUT = 64;  // doubles of the pinned result block
 
 struct Buf {
     void* p = nullptr;
@@ -61,6 +62,7 @@ struct bounce_ctx {
     int hist_alloc = 0;
     long long* d_step = nullptr;
     int* h_err = nullptr;        // pinned
+    double* h_out = nullptr;     // pinned [H_OUT]: results of a call on their way to the host
     double* h_stage = nullptr;   // pinned [6 n]: interleaved q then v on their way to or from the device
     double* d_stage = nullptr;   // device [6 n]
     unsigned long long* h_cnt = nullptr;
@@ -105,6 +107,7 @@ struct bounce_ctx {
     int4* tile_items = nullptr;
     int tile_cap = 0;
     std::vector<int> rep_bounds;  // [replicas + 1] atom ranges for the tiles ({0, n} for one system)
+    double rate_sum = -1.0;       // expected_proposals: its sum over the atoms (< 0: to be made)
     bool lite_jumps = false;      // BOUNCE integrators take the thread-per-atom step kernel
 };
 
@@ -458,10 +461,56 @@ void fill_params(bounce_ctx* c, const std::vector<double>& sig, const std::vecto
     p.key1 = (uint32_t)(g.seed >> 32);
 }
 
+// Bounds of n positions (interleaved).
+struct HostBox {
+    double lo[3], hi[3];
+};
+HostBox host_box(const double* q, int n) {
+    HostBox b;
+    for (int d = 0; d < 3; ++d) b.lo[d] = b.hi[d] = q[d];
+    for (int i = 1; i < n; ++i)
+        for (int d = 0; d < 3; ++d) {
+            const double x = q[3 * (size_t)i + d];
+            b.lo[d] = x < b.lo[d] ? x : b.lo[d];
+            b.hi[d] = x > b.hi[d] ? x : b.hi[d];
+        }
+    return b;
+}
+
+// Whether all of x[0..n) is finite: x 0 is NaN for an infinity or a NaN, and
+// eight sums keep the loop free of a dependent chain.
+bool all_finite(const double* x, size_t n) {
+    double s[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    size_t k = 0;
+    for (; k + 8 <= n; k += 8)
+        for (int u = 0; u < 8; ++u) s[u] += x[k + u] * 0.0;
+    for (; k < n; ++k) s[0] += x[k] * 0.0;
+    return ((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7])) == 0.0;
+}
+
+// Most atoms of one column of an ncx x ncy grid (as the device bins them).
+int fullest_column(const bounce_config& g, const double* q, int n, int ncx, int ncy, double ox, double oy, double ihx,
+                   double ihy) {
+    std::vector<int> cnt((size_t)ncx * ncy, 0);
+    const double iLx = g.periodic ? 1.0 / g.box[0] : 0.0, iLy = g.periodic ? 1.0 / g.box[1] : 0.0;
+    int mx = 0;
+    for (int i = 0; i < n; ++i) {
+        double x = q[3 * (size_t)i], y = q[3 * (size_t)i + 1];
+        if (g.periodic) {
+            x -= g.box[0] * std::floor(x * iLx);
+            y -= g.box[1] * std::floor(y * iLy);
+        }
+        const int cx = std::min(std::max((int)std::floor((x - ox) * ihx), 0), ncx - 1);
+        const int cy = std::min(std::max((int)std::floor((y - oy) * ihy), 0), ncy - 1);
+        mx = std::max(mx, ++cnt[(size_t)cy * ncx + cx]);
+    }
+    return mx;
+}
+
 // Cell grid for the current host positions: cells of edge >= r_list / 3
 // (the row builder scans, for each (y, z) cell row within reach, only the
 // x-span of cells the r_list sphere can touch).
-int setup_grid(bounce_ctx* c, const double* q) {
+int setup_grid(bounce_ctx* c, const HostBox& hb) {
     DevSys& s = c->ds;
     const double rl = r_list(c->cfg);
     const double reach = std::isfinite(rl) ? rl * (1.0 + 1e-5) + 1e-3 : INFINITY;
@@ -477,13 +526,7 @@ int setup_grid(bounce_ctx* c, const double* q) {
             h = Lb / nc[d];
             ih[d] = (float)(nc[d] / Lb);
         } else {
-            double lo = 1e300, hi = -1e300;
-            for (int i = 0; i < c->n; ++i) {
-                lo = std::min(lo, q[3 * i + d]);
-                hi = std::max(hi, q[3 * i + d]);
-            }
-            lo -= 5.0;
-            hi += 5.0;
+            const double lo = hb.lo[d] - 5.0, hi = hb.hi[d] + 5.0;
             const double ext = hi - lo;
             if (std::isfinite(edge_min)) {
                 h = std::max(edge_min, ext / 256.0);
@@ -533,7 +576,7 @@ int setup_grid(bounce_ctx* c, const double* q) {
 #define CL_PRUNE_SKIN 0.8
 #endif
 
-int setup_clusters(bounce_ctx* c, const double* q) {
+int setup_clusters(bounce_ctx* c, const double* q, const HostBox& hb) {
     DevClu& k = c->ds.cl;
     const bounce_config& g = c->cfg;
     const int n = c->n;
@@ -551,12 +594,8 @@ int setup_clusters(bounce_ctx* c, const double* q) {
             lo[d] = 0.0;
             hi[d] = g.box[d];
         } else {
-            lo[d] = 1e300;
-            hi[d] = -1e300;
-            for (int i = 0; i < n; ++i) {
-                lo[d] = std::min(lo[d], q[3 * i + d]);
-                hi[d] = std::max(hi[d], q[3 * i + d]);
-            }
+            lo[d] = hb.lo[d];
+            hi[d] = hb.hi[d];
         }
     }
     // keep the current grid (a periodic box's is fixed; a droplet's while
@@ -564,18 +603,7 @@ int setup_clusters(bounce_ctx* c, const double* q) {
     if (k.on && !c->cl_force) {
         const double x0 = k.ox, y0 = k.oy, x1 = k.ox + k.ncx / k.ihx, y1 = k.oy + k.ncy / k.ihy;
         if (g.periodic || (lo[0] >= x0 && lo[1] >= y0 && hi[0] <= x1 && hi[1] <= y1)) {
-            std::vector<int> cnt(k.ncol, 0);
-            int mx = 0;
-            for (int i = 0; i < n; ++i) {
-                double x = q[3 * i], y = q[3 * i + 1];
-                if (g.periodic) {
-                    x -= g.box[0] * std::floor(x / g.box[0]);
-                    y -= g.box[1] * std::floor(y / g.box[1]);
-                }
-                const int cx = std::min(std::max((int)std::floor((x - x0) * k.ihx), 0), k.ncx - 1);
-                const int cy = std::min(std::max((int)std::floor((y - y0) * k.ihy), 0), k.ncy - 1);
-                mx = std::max(mx, ++cnt[cy * k.ncx + cx]);
-            }
+            const int mx = fullest_column(g, q, n, k.ncx, k.ncy, x0, y0, k.ihx, k.ihy);
             if (4 * mx <= 3 * k.maxcol) return BOUNCE_OK;
         }
     }
@@ -606,18 +634,7 @@ int setup_clusters(bounce_ctx* c, const double* q) {
     nk.oy = g.periodic ? 0.f : (float)lo[1];
     nk.ihx = (float)(nc[0] / (hi[0] - lo[0]));
     nk.ihy = (float)(nc[1] / (hi[1] - lo[1]));
-    std::vector<int> cnt(nk.ncol, 0);
-    int mx = 0;
-    for (int i = 0; i < n; ++i) {
-        double x = q[3 * i], y = q[3 * i + 1];
-        if (g.periodic) {
-            x -= g.box[0] * std::floor(x / g.box[0]);
-            y -= g.box[1] * std::floor(y / g.box[1]);
-        }
-        const int cx = std::min(std::max((int)std::floor((x - nk.ox) * nk.ihx), 0), nk.ncx - 1);
-        const int cy = std::min(std::max((int)std::floor((y - nk.oy) * nk.ihy), 0), nk.ncy - 1);
-        mx = std::max(mx, ++cnt[cy * nk.ncx + cx]);
-    }
+    const int mx = fullest_column(g, q, n, nk.ncx, nk.ncy, nk.ox, nk.oy, nk.ihx, nk.ihy);
     const int want = (mx * 3 / 2 + 16 + 7) / 8 * 8;
     if (mx > BOUNCE_CL_MAXCOL) return fail(c, BOUNCE_ERR_UNSUPPORTED, "a cluster column holds more than 1024 atoms");
     nk.maxcol = std::min(want, BOUNCE_CL_MAXCOL);
@@ -739,14 +756,6 @@ int setup_tiles(bounce_ctx* c) {
     T.pairs = pairs ? 1 : 0;
     T.blocks = c->tile_blocks;
     drop_graphs(c);
-    return BOUNCE_OK;
-}
-
-// Raise the cluster rebuild flag (positions were replaced).
-int flag_clusters(bounce_ctx* c, cudaStream_t st) {
-    if (!c->ds.cl.on) return BOUNCE_OK;
-    static const int one = 1;
-    CU(cudaMemcpyAsync(c->ds.cl.rebuild, &one, sizeof(int), cudaMemcpyHostToDevice, st));
     return BOUNCE_OK;
 }
 
@@ -951,28 +960,30 @@ DevSys run_view(const bounce_ctx* c, int integ) {
 // lower it).  On 64 droplets of 64-1,024 molecules, LJ on the jumps (0.13
 // proposals per atom-step), the thread-per-atom kernel that this admits takes
 // 39 us where the cooperative one takes 117.
-double expected_proposals(const bounce_ctx* c, double rho) {
+double expected_proposals(bounce_ctx* c, double rho) {
     const bounce_config& g = c->cfg;
-    const double beta = 1.0 / (KB_D * g.temperature_K);
     const double rl = r_list(g);
-    const double nball = std::isfinite(rl) ? rho * 4.18879 * rl * rl * rl : INFINITY;
-    // jump rows that keep only the jump partners: the share of the atoms of a partner type
-    double share[BOUNCE_MAXT];
-    for (int a = 0; a < BOUNCE_MAXT; ++a) {
-        int k = 0;
-        if (c->jfilter)
-            for (int i = 0; i < c->n; ++i) k += (c->pp.jpart[a] >> c->type[i]) & 1;
-        share[a] = c->jfilter && c->n ? (double)k / c->n : 1.0;
+    if (c->rate_sum < 0.0) {  // per partner (with a cutoff), or with the replica's atoms as partners
+        const double beta = 1.0 / (KB_D * g.temperature_K);
+        // jump rows that keep only the jump partners: the share of the atoms of a partner type
+        double share[BOUNCE_MAXT];
+        for (int a = 0; a < BOUNCE_MAXT; ++a) {
+            int k = 0;
+            if (c->jfilter)
+                for (int i = 0; i < c->n; ++i) k += (c->pp.jpart[a] >> c->type[i]) & 1;
+            share[a] = c->jfilter && c->n ? (double)k / c->n : 1.0;
+        }
+        double sum = 0.0;
+        size_t rep = 0;
+        for (int i = 0; i < c->n; ++i) {
+            while (i >= c->rep_bounds[rep + 1]) ++rep;
+            const double partners = std::isfinite(rl) ? 1.0 : (double)(c->rep_bounds[rep + 1] - c->rep_bounds[rep]);
+            const double vbar = std::sqrt(8.0 * KB_D * g.temperature_K * ACCEL_D / (M_PI * c->mass[i]));
+            sum += beta * vbar * c->Lstar[c->type[i]] * partners * share[c->type[i]] * g.dt_fs;
+        }
+        c->rate_sum = sum / c->n;
     }
-    double sum = 0.0;
-    size_t rep = 0;
-    for (int i = 0; i < c->n; ++i) {
-        while (i >= c->rep_bounds[rep + 1]) ++rep;
-        const double nbar = std::min((double)(c->rep_bounds[rep + 1] - c->rep_bounds[rep]), nball);
-        const double vbar = std::sqrt(8.0 * KB_D * g.temperature_K * ACCEL_D / (M_PI * c->mass[i]));
-        sum += beta * vbar * c->Lstar[c->type[i]] * nbar * share[c->type[i]] * g.dt_fs;
-    }
-    return sum / c->n;
+    return std::isfinite(rl) ? c->rate_sum * std::min((double)c->n, rho * 4.18879 * rl * rl * rl) : c->rate_sum;
 }
 
 // The gated rebuilds at one step boundary: the clusters (their own flag) and
@@ -1105,6 +1116,7 @@ int bounce_create(bounce_ctx** out, const bounce_config* cfg) {
     }
     if (cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaMallocHost(&c->h_err, sizeof(int)) != cudaSuccess ||
+        cudaMallocHost(&c->h_out, H_OUT * sizeof(double)) != cudaSuccess ||
         cudaMallocHost(&c->h_cnt, CNT_N * sizeof(unsigned long long)) != cudaSuccess) {
         delete c;
         return BOUNCE_ERR_CUDA;
@@ -1265,6 +1277,7 @@ int bounce_set_lj(bounce_ctx* c, int32_t T, const double* sigma, const double* e
             ep[a * c->n_types + b] = eps[a * T + b];
         }
     compute_bounds(c, sg, ep);
+    c->rate_sum = -1.0;
     fill_params(c, sg, ep);
     set_jump_partners(c, sg, ep);
     drop_graphs(c);
@@ -1312,25 +1325,20 @@ int bounce_set_state(bounce_ctx* c, const double* q, const double* v, int64_t st
         hq = c->h_stage;
         hv = c->h_stage + n3;
     }
-    for (size_t k = 0; k < n3; ++k)
-        if (!std::isfinite(hq[k]) || !std::isfinite(hv[k]))
-            return fail(c, BOUNCE_ERR_NONFINITE, "non-finite position or velocity");
+    if (!all_finite(hq, n3) || !all_finite(hv, n3))
+        return fail(c, BOUNCE_ERR_NONFINITE, "non-finite position or velocity");
     // short rows (systems without a cutoff) need one row-builder window over every atom
     if (!c->ds.rep_of && c->pp.rshort2 < INFINITY && c->bitmap_warps < (c->n + 31) / 32)
         return fail(c, BOUNCE_ERR_UNSUPPORTED, "too many atoms for short rows without a cutoff");
     const DevSys before = c->ds;
-    int r = setup_grid(c, hq);
+    const HostBox hb = host_box(hq, n);
+    int r = setup_grid(c, hb);
     if (r) return r;
-    if ((r = setup_clusters(c, hq))) return r;
+    if ((r = setup_clusters(c, hq, hb))) return r;
     {
         // density for the rate estimate: the box, or half the droplet's bounding box
-        double lo[3] = {1e300, 1e300, 1e300}, hi[3] = {-1e300, -1e300, -1e300}, vol = 1.0;
-        for (int i = 0; i < c->n; ++i)
-            for (int d = 0; d < 3; ++d) {
-                lo[d] = std::min(lo[d], hq[3 * i + d]);
-                hi[d] = std::max(hi[d], hq[3 * i + d]);
-            }
-        for (int d = 0; d < 3; ++d) vol *= c->cfg.periodic ? c->cfg.box[d] : std::max(hi[d] - lo[d], 1.0);
+        double vol = 1.0;
+        for (int d = 0; d < 3; ++d) vol *= c->cfg.periodic ? c->cfg.box[d] : std::max(hb.hi[d] - hb.lo[d], 1.0);
         const double rho = c->n / (c->cfg.periodic ? vol : 0.55 * vol);
         const bool lite = expected_proposals(c, rho) < 0.5;
         if (lite != c->lite_jumps) drop_graphs(c);
@@ -1356,23 +1364,12 @@ int bounce_set_state(bounce_ctx* c, const double* q, const double* v, int64_t st
         dq = c->d_stage;
         dv = c->d_stage + n3;
     }
-    launch_state_in(s, dq, dv, cur, st);
-    long long st0 = step;
-    CU(cudaMemcpyAsync(c->d_step, &st0, sizeof(long long), cudaMemcpyHostToDevice, st));
-    launch_pack_positions(s, c->pp, cur, st);
     // rows stay valid while every atom is within skin/2 of where they were
     // built (the same test as during a run); otherwise the next launch
     // rebuilds them
-    if (c->rows_valid) {
-        launch_flag_moved(s, c->pp, cur, st);
-    } else {
-        const int one = 1;
-        CU(cudaMemcpyAsync(s.rebuild, &one, sizeof(int), cudaMemcpyHostToDevice, st));
-        c->rows_valid = true;
-    }
-    if ((r = flag_clusters(c, st))) return r;
+    launch_state_in(s, c->pp, dq, dv, cur, step, c->rows_valid ? 1 : 2, st);
+    c->rows_valid = true;
     c->rows_check_due = false;
-    CU(cudaMemsetAsync(s.err, 0, sizeof(int), st));
     CU(cudaStreamSynchronize(st));
     c->step0 = step;
     c->cur_step = step;
@@ -1597,13 +1594,14 @@ int bounce_autotune(bounce_ctx* c, int32_t integ, void* stream, bounce_tuning* o
         // cluster columns: edge factor around (8 / density)^(1/3)
         std::vector<double> q(3 * (size_t)c->n);
         if ((r = bounce_get_state(c, q.data(), nullptr, BOUNCE_HOST, stream))) return r;
+        const HostBox hb = host_box(q.data(), c->n);
         const double fs[5] = {0.8, 0.9, 1.0, 1.12, 1.25};
         double best = 1e30, bf = c->cl_edge_factor;
         const int list = (part == 3 && c->ds.cl.nlists > 1) ? 1 : 0;
         for (double f : fs) {
             c->cl_edge_factor = f;
             c->cl_force = true;
-            if ((r = setup_clusters(c, q.data()))) break;
+            if ((r = setup_clusters(c, q.data(), hb))) break;
             launch_cluster_rebuild(c->ds, c->pp, 0, true, st);
             const double ms = time_pairs([&] { launch_cluster_pairs(c->ds, c->pp, 0, part, list, st); });
             ++out->candidates;
@@ -1614,7 +1612,7 @@ int bounce_autotune(bounce_ctx* c, int32_t integ, void* stream, bounce_tuning* o
         }
         c->cl_edge_factor = bf;
         c->cl_force = true;
-        if (!r) r = setup_clusters(c, q.data());
+        if (!r) r = setup_clusters(c, q.data(), hb);
         if (!r) launch_cluster_rebuild(c->ds, c->pp, 0, true, st);
         const size_t ns = (size_t)c->ds.cl.ncol * c->ds.cl.maxcl * BOUNCE_CL;
         CU(cudaMemsetAsync(c->ds.cl.acc, 0, 3 * ns * sizeof(unsigned long long), st));
@@ -1657,12 +1655,11 @@ int bounce_get_energies(bounce_ctx* c, bounce_energies* out, void* stream) {
     if (!c->have_state) return fail(c, BOUNCE_ERR_STATE, "no state");
     cudaSetDevice(c->cfg.device);
     cudaStream_t st = (cudaStream_t)stream;
-    long long step;
-    CU(cudaMemcpyAsync(&step, c->d_step, sizeof(long long), cudaMemcpyDeviceToHost, st));
-    CU(cudaStreamSynchronize(st));
+    const long long step = c->cur_step;
     if (int r0 = prepare_readers(c, st)) return r0;
     launch_energies(c->ds, c->pp, (int)(step & 1), c->terms, st);
-    double tot[5], pe[2] = {0.0, 0.0};
+    double *tot = c->h_out, *pe = c->h_out + 5;
+    pe[0] = pe[1] = 0.0;
     if (c->has_pme) {
         launch_pme(c->ds, c->pp, c->pme, 0, st, true);
         launch_pme_energy(c->pme, c->n, c->terms + 6 * (size_t)c->n + 1024, st);
@@ -1670,7 +1667,6 @@ int bounce_get_energies(bounce_ctx* c, bounce_energies* out, void* stream) {
     }
     CU(cudaMemcpyAsync(tot, c->terms + 5 * (size_t)c->n, 5 * sizeof(double), cudaMemcpyDeviceToHost, st));
     CU(cudaMemcpyAsync(c->h_cnt, c->ds.cnt, CNT_N * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
-    CU(cudaStreamSynchronize(st));
     int r = check_err(c, st);
     if (r) return r;
     out->coulomb = KCOUL_D / (double)c->pp.kcoul * tot[0];
@@ -1705,14 +1701,11 @@ int bounce_pair_histogram(bounce_ctx* c, int32_t ta, int32_t tb, double r_max, i
         if (r) return r;
         c->hist_alloc = n_bins;
     }
-    long long step;
-    CU(cudaMemcpyAsync(&step, c->d_step, sizeof(long long), cudaMemcpyDeviceToHost, st));
-    CU(cudaStreamSynchronize(st));
+    const long long step = c->cur_step;
     if (int r0 = prepare_readers(c, st)) return r0;
     CU(cudaMemsetAsync(c->hist, 0, n_bins * sizeof(unsigned long long), st));
     launch_pair_hist(c->ds, c->pp, (int)(step & 1), ta, tb, r_max, n_bins, c->hist, st);
     CU(cudaMemcpyAsync(hist, c->hist, n_bins * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-    CU(cudaStreamSynchronize(st));
     return check_err(c, st);
 }
 
@@ -1725,9 +1718,7 @@ int bounce_set_msd_reference(bounce_ctx* c, void* stream) {
         int r = dalloc(c, &c->msd_ref, 3 * (size_t)c->n);
         if (r) return r;
     }
-    long long step;
-    CU(cudaMemcpyAsync(&step, c->d_step, sizeof(long long), cudaMemcpyDeviceToHost, st));
-    CU(cudaStreamSynchronize(st));
+    const long long step = c->cur_step;
     const int cur = (int)(step & 1);
     const size_t b = c->n * sizeof(double);
     CU(cudaMemcpyAsync(c->msd_ref, c->ds.qx[cur], b, cudaMemcpyDeviceToDevice, st));
@@ -1743,9 +1734,7 @@ int bounce_msd(bounce_ctx* c, int32_t type, double* out, void* stream) {
     if (!c->have_msd_ref) return fail(c, BOUNCE_ERR_STATE, "no msd reference");
     cudaSetDevice(c->cfg.device);
     cudaStream_t st = (cudaStream_t)stream;
-    long long step;
-    CU(cudaMemcpyAsync(&step, c->d_step, sizeof(long long), cudaMemcpyDeviceToHost, st));
-    CU(cudaStreamSynchronize(st));
+    const long long step = c->cur_step;
     launch_msd(c->ds, c->msd_ref, c->msd_ref + c->n, c->msd_ref + 2 * (size_t)c->n, (int)(step & 1), type, c->terms,
                st);
     double tot[2];
@@ -1780,17 +1769,15 @@ int bounce_compute_gradient(bounce_ctx* c, int32_t part, double* grad, int32_t w
     if (!c->have_state) return fail(c, BOUNCE_ERR_STATE, "no state");
     cudaSetDevice(c->cfg.device);
     cudaStream_t st = (cudaStream_t)stream;
-    long long step;
-    CU(cudaMemcpyAsync(&step, c->d_step, sizeof(long long), cudaMemcpyDeviceToHost, st));
-    CU(cudaStreamSynchronize(st));
+    const long long step = c->cur_step;
     if (int r0 = prepare_readers(c, st)) return r0;
     const cudaMemcpyKind kind = where == BOUNCE_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
     if (part == BOUNCE_GRAD_RECIP) {
         if (!c->has_pme) return fail(c, BOUNCE_ERR_STATE, "no SPME grid configured");
         launch_pme(c->ds, c->pp, c->pme, 0, st);
-        for (int d = 0; d < 3; ++d)
-            CU(cudaMemcpy2DAsync(grad + d, 3 * sizeof(double), c->pme.grad + (size_t)d * c->n, sizeof(double),
-                                 sizeof(double), c->n, kind, st));
+        double* out = where == BOUNCE_DEVICE ? grad : c->terms;
+        launch_soa_out(c->n, c->pme.grad, out, st);
+        if (where == BOUNCE_HOST) CU(cudaMemcpyAsync(grad, out, 3 * (size_t)c->n * sizeof(double), kind, st));
     } else if (c->ds.tl.on && (part == BOUNCE_GRAD_FULL || (part == BOUNCE_GRAD_SHORT && !(c->pp.rshort2 < INFINITY)))) {
         // bonded terms, then the all-pairs tile sums added (the run's kernels)
         double* out = c->terms;
@@ -1812,7 +1799,6 @@ int bounce_compute_gradient(bounce_ctx* c, int32_t part, double* grad, int32_t w
         launch_gradient(c->ds, c->pp, part, (int)(step & 1), out, st);
         CU(cudaMemcpyAsync(grad, out, 3 * (size_t)c->n * sizeof(double), kind, st));
     }
-    CU(cudaStreamSynchronize(st));
     return check_err(c, st);
 }
 
@@ -1823,9 +1809,7 @@ int bounce_jump_half(bounce_ctx* c, int64_t step, int32_t stream_id, int32_t* M,
     if (!c->have_state) return fail(c, BOUNCE_ERR_STATE, "no state");
     cudaSetDevice(c->cfg.device);
     cudaStream_t st = (cudaStream_t)stream;
-    long long cur_step;
-    CU(cudaMemcpyAsync(&cur_step, c->d_step, sizeof(long long), cudaMemcpyDeviceToHost, st));
-    CU(cudaStreamSynchronize(st));
+    const long long cur_step = c->cur_step;
     if (c->jfilter) {
         // the stand-alone half-step draws over the full rows
         if (int r0 = prepare_readers(c, st)) return r0;
@@ -1843,7 +1827,6 @@ int bounce_jump_half(bounce_ctx* c, int64_t step, int32_t stream_id, int32_t* M,
     const cudaMemcpyKind kind = where == BOUNCE_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
     if (M) CU(cudaMemcpyAsync(M, dM, c->n * sizeof(int), kind, st));
     if (nacc) CU(cudaMemcpyAsync(nacc, dA, c->n * sizeof(int), kind, st));
-    CU(cudaStreamSynchronize(st));
     return check_err(c, st);
 }
 
@@ -1909,6 +1892,7 @@ int bounce_set_replicas(bounce_ctx* c, int32_t n_rep, const int32_t* off, const 
     c->ds.rep_off = doff;
     c->ds.rep_key = dkey;
     c->rep_bounds.assign(off, off + n_rep + 1);
+    c->rate_sum = -1.0;
     if ((rr = setup_tiles(c))) return rr;
     drop_graphs(c);
     c->rows_valid = false;
@@ -1946,14 +1930,7 @@ int bounce_pair_forward(bounce_ctx* c, const double* q, int32_t T, const double*
     const int cur = (int)(c->cur_step & 1);
     const int n = c->n;
     if (q) {
-        CU(cudaMemcpy2DAsync(c->ds.qx[cur], sizeof(double), q + 0, 3 * sizeof(double), sizeof(double), n,
-                             cudaMemcpyDeviceToDevice, st));
-        CU(cudaMemcpy2DAsync(c->ds.qy[cur], sizeof(double), q + 1, 3 * sizeof(double), sizeof(double), n,
-                             cudaMemcpyDeviceToDevice, st));
-        CU(cudaMemcpy2DAsync(c->ds.qz[cur], sizeof(double), q + 2, 3 * sizeof(double), sizeof(double), n,
-                             cudaMemcpyDeviceToDevice, st));
-        launch_pack_positions(c->ds, c->pp, cur, st);
-        if ((r = flag_clusters(c, st))) return r;
+        launch_state_in(c->ds, c->pp, q, nullptr, cur, -1, 0, st);
         if ((r = prepare_readers(c, st, true))) return r;
     } else {
         if ((r = prepare_readers(c, st))) return r;
@@ -1961,11 +1938,10 @@ int bounce_pair_forward(bounce_ctx* c, const double* q, int32_t T, const double*
     double* eatom = c->terms;
     double* esum = c->terms + 6 * (size_t)n + 1024;
     launch_pair_forward(c->ds, c->pp, fq, fs, fe, T, cur, forces, eatom, esum, st);
-    double e = 0.0;
-    CU(cudaMemcpyAsync(&e, esum, sizeof(double), cudaMemcpyDeviceToHost, st));
-    CU(cudaStreamSynchronize(st));
-    if (energy) *energy = e;
-    return check_err(c, st);
+    CU(cudaMemcpyAsync(c->h_out, esum, sizeof(double), cudaMemcpyDeviceToHost, st));
+    r = check_err(c, st);
+    if (energy) *energy = c->h_out[0];
+    return r;
 }
 
 int bounce_pair_backward(bounce_ctx* c, int32_t T, const double* qt, const double* sig, const double* eps,
@@ -2009,6 +1985,7 @@ void bounce_destroy(bounce_ctx* c) {
     free_all(c);
     if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
     if (c->h_err) cudaFreeHost(c->h_err);
+    if (c->h_out) cudaFreeHost(c->h_out);
     if (c->h_cnt) cudaFreeHost(c->h_cnt);
     delete c;
 }

@@ -185,7 +185,7 @@ struct DevPme {
     const float* bc;             // influence function B(m) C(m)
     float4* frac;                // [n] grid fractions of each atom, w: its grid point, 10 bits an axis (spread -> gather)
     double* grad;                // [3 n] SoA gradient of E_recip + E_excl
-    double* eexcl;               // [n] exclusion energy per atom (pairs j > i)
+    double* eexcl;               // [n] exclusion energy partials (one per CTA of the kernel that makes them)
     double* eterm;               // [256] energy partials of the convolution
     const int* ex_off;           // [n + 1] same-molecule partners of each atom
     const int* ex_idx;
@@ -670,8 +670,9 @@ void launch_jump_half(const DevSys& s, const Params& p, int cur, long long step,
                       cudaStream_t st);
 void launch_energies(const DevSys& s, const Params& p, int cur, double* terms, cudaStream_t st);
 void launch_advance_step(const DevSys& s, long long by, cudaStream_t st);
-void launch_pack_positions(const DevSys& s, const Params& p, int cur, cudaStream_t st);
-void launch_state_in(const DevSys& s, const double* q, const double* v, int cur, cudaStream_t st);
+void launch_state_in(const DevSys& s, const Params& p, const double* q, const double* v, int cur, long long step, int rows,
+                     cudaStream_t st);
+void launch_soa_out(int n, const double* g, double* out, cudaStream_t st);
 void launch_state_out(const DevSys& s, double* q, double* v, cudaStream_t st);
 // Raises the rebuild flag when an atom at positions `cur` lies more than
 // skin/2 from its position at the last row build (the step kernel's test).

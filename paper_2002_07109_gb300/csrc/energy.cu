@@ -1,5 +1,5 @@
 // Energies of the current state (unsplit W, paper Sec. IV.A / V) and the
-// position packing used after a state upload.
+// state on its way in and out.
 //
 // Pair energies: one warp per atom sums W over the members j > i of its row
 // with r < r_c (FP32 per pair, FP32 per lane, FP64 across lanes); bonded and
@@ -109,25 +109,6 @@ __global__ void k_sum_pass2(const double* partial, double* out) {
     if (threadIdx.x < T) out[threadIdx.x] = part[threadIdx.x][0];
 }
 
-// Split FP32 copies (hi + lo) of the FP64 positions of buffer `cur`;
-// positions are wrapped into the box for periodic systems.
-__global__ void k_pack(DevSys s, Params p, int cur) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < s.n; i += gridDim.x * blockDim.x) {
-        double x = s.qx[cur][i], y = s.qy[cur][i], z = s.qz[cur][i];
-        if (p.periodic) {
-            x = wrap_box(x, p.Ld[0], p.iLd[0]);
-            y = wrap_box(y, p.Ld[1], p.iLd[1]);
-            z = wrap_box(z, p.Ld[2], p.iLd[2]);
-        }
-        const float hx = __double2float_rn(x), hy = __double2float_rn(y), hz = __double2float_rn(z);
-        const float4 oh = s.phi[cur][i];
-        const float4 ol = s.plo[cur][i];
-        s.phi[cur][i] = make_float4(hx, hy, hz, oh.w);
-        s.plo[cur][i] = make_float4(__double2float_rn(x - (double)hx), __double2float_rn(y - (double)hy),
-                                    __double2float_rn(z - (double)hz), ol.w);
-    }
-}
-
 }  // namespace
 
 void launch_energies(const DevSys& s, const Params& p, int cur, double* terms, cudaStream_t st) {
@@ -140,16 +121,53 @@ void launch_energies(const DevSys& s, const Params& p, int cur, double* terms, c
     k_sum_pass2<5><<<1, SUM_CTAS, 0, st>>>(partial, terms + 5 * (size_t)s.n);
 }
 
-// State in: interleaved q[n][3], v[n][3] (device) -> FP64 SoA at buffer cur.
-__global__ void k_state_in(DevSys s, const double* q, const double* v, int cur) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < s.n; i += gridDim.x * blockDim.x) {
-        s.qx[cur][i] = q[3 * (size_t)i];
-        s.qy[cur][i] = q[3 * (size_t)i + 1];
-        s.qz[cur][i] = q[3 * (size_t)i + 2];
+// State in: interleaved q[n][3] and v[n][3] (device; v may be null: kept) ->
+// FP64 SoA at buffer cur and its split FP32 copies, wrapped into the box, and
+// what a new state sets: the step counter and the error bits (step >= 0), the
+// rows' rebuild flag (rows 1: raised where an atom lies more than skin/2 from
+// its position at the last build -- the step kernel's test; 2: raised) and
+// the clusters' flag.  One launch in place of six copies and kernels.
+__global__ void k_state_in(DevSys s, Params p, const double* q, const double* v, int cur, long long step, int rows) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0) {
+        if (step >= 0) {
+            *const_cast<long long*>(s.step_base) = step;
+            *s.err = 0;
+        }
+        if (rows == 2) *s.rebuild = 1;
+        if (s.cl.on) *s.cl.rebuild = 1;
+    }
+    if (i >= s.n) return;
+    double x = q[3 * (size_t)i], y = q[3 * (size_t)i + 1], z = q[3 * (size_t)i + 2];
+    s.qx[cur][i] = x;
+    s.qy[cur][i] = y;
+    s.qz[cur][i] = z;
+    if (v) {
         s.vx[i] = v[3 * (size_t)i];
         s.vy[i] = v[3 * (size_t)i + 1];
         s.vz[i] = v[3 * (size_t)i + 2];
     }
+    if (rows == 1) {
+        const double ex = x - s.refx[i], ey = y - s.refy[i], ez = z - s.refz[i];
+        if (((s.rows_move >> s.type[i]) & 1) && ex * ex + ey * ey + ez * ez > p.skin_half2) atomicOr(s.rebuild, 1);
+    }
+    if (p.periodic) {
+        x = wrap_box(x, p.Ld[0], p.iLd[0]);
+        y = wrap_box(y, p.Ld[1], p.iLd[1]);
+        z = wrap_box(z, p.Ld[2], p.iLd[2]);
+    }
+    const float hx = __double2float_rn(x), hy = __double2float_rn(y), hz = __double2float_rn(z);
+    s.phi[cur][i] = make_float4(hx, hy, hz, s.phi[cur][i].w);
+    s.plo[cur][i] = make_float4(__double2float_rn(x - (double)hx), __double2float_rn(y - (double)hy),
+                                __double2float_rn(z - (double)hz), s.plo[cur][i].w);
+}
+
+// Gradient out: SoA [3 n] -> interleaved [n][3].
+__global__ void k_soa_out(int n, const double* g, double* out) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= 3 * n) return;
+    const int i = t / 3;
+    out[t] = g[(size_t)(t - 3 * i) * n + i];
 }
 
 // State out: FP64 SoA of the current step (read on the device) -> interleaved
@@ -170,14 +188,15 @@ __global__ void k_state_out(DevSys s, double* q, double* v) {
     }
 }
 
-void launch_state_in(const DevSys& s, const double* q, const double* v, int cur, cudaStream_t st) {
-    k_state_in<<<(s.n + 255) / 256, 256, 0, st>>>(s, q, v, cur);
+void launch_state_in(const DevSys& s, const Params& p, const double* q, const double* v, int cur, long long step, int rows,
+                     cudaStream_t st) {
+    k_state_in<<<(s.n + 255) / 256, 256, 0, st>>>(s, p, q, v, cur, step, rows);
+}
+
+void launch_soa_out(int n, const double* g, double* out, cudaStream_t st) {
+    k_soa_out<<<(3 * n + 255) / 256, 256, 0, st>>>(n, g, out);
 }
 
 void launch_state_out(const DevSys& s, double* q, double* v, cudaStream_t st) {
     k_state_out<<<(s.n + 255) / 256, 256, 0, st>>>(s, q, v);
-}
-
-void launch_pack_positions(const DevSys& s, const Params& p, int cur, cudaStream_t st) {
-    k_pack<<<(s.n + 255) / 256, 256, 0, st>>>(s, p, cur);
 }

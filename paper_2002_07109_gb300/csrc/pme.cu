@@ -450,14 +450,17 @@ __global__ void __launch_bounds__(128) k_pme_gather(DevSys s, Params p, DevPme m
     m.grad[2 * (size_t)s.n + i] = Gz;
 }
 
-// Exclusion energy -k q_i q_j erf(beta r)/r of the pairs (i, j > i) owned by
-// atom i (for bounce_get_energies).
-__global__ void k_pme_excl(DevSys s, Params p, DevPme m, int step_off) {
+// Exclusion energies -k q_i q_j erf(beta r)/r of the pairs (i, j > i) owned by
+// the CTA's atoms, summed in a fixed order into eexcl[CTA].
+constexpr int EXCL_NT = 128;
+__global__ void __launch_bounds__(EXCL_NT) k_pme_excl(DevSys s, Params p, DevPme m, int step_off) {
     chain_enter();
+    __shared__ double red[EXCL_NT];
     const int cur = (int)((*s.step_base + step_off) & 1);
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < s.n; i += gridDim.x * blockDim.x) {
+    const int i = blockIdx.x * EXCL_NT + threadIdx.x;
+    double ex = 0.0;
+    if (i < s.n) {
         const float4 hi = s.phi[cur][i], lo = s.plo[cur][i];
-        double ex = 0.0;
         for (int t = m.ex_off[i]; t < m.ex_off[i + 1]; ++t) {
             const int j = m.ex_idx[t];
             if (j <= i) continue;
@@ -467,8 +470,14 @@ __global__ void k_pme_excl(DevSys s, Params p, DevPme m, int step_off) {
             const float qq = (float)KCOUL_D * hi.w * hj.w;
             ex += -(double)qq * (double)(erff(m.beta * r) / r);
         }
-        m.eexcl[i] = ex;
     }
+    red[threadIdx.x] = ex;
+    __syncthreads();
+    for (int w = EXCL_NT / 2; w > 0; w >>= 1) {
+        if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) m.eexcl[blockIdx.x] = red[0];
 }
 
 // Lines of K = 32 M points (M = 1..5): one warp per line, no shared-memory
@@ -974,6 +983,7 @@ __global__ void k_pme_real(DevPme m) {
     }
 }
 
+// Sums of the convolution's partials and of the n partials of the exclusions.
 __global__ void k_pme_energy_sum(DevPme m, int nparts, int n, double* out) {
     __shared__ double red[2][256];
     double a = 0.0, b = 0.0;
@@ -1143,7 +1153,7 @@ void launch_pme(const DevSys& s, const Params& p, const DevPme& m, int step_off,
         // the energy partials need no potential: no way back, no gather
         transform(0, -1.f);
         launch_chained(k_pme_convolve<true>, PME_CONV_CTAS, 256, 0, st, m);
-        launch_chained(k_pme_excl, nb, tb, 0, st, s, p, m, step_off);
+        launch_chained(k_pme_excl, (s.n + EXCL_NT - 1) / EXCL_NT, EXCL_NT, 0, st, s, p, m, step_off);
         return;
     }
     if (pl.kind == PME_WARP) {
@@ -1176,5 +1186,5 @@ void launch_pme(const DevSys& s, const Params& p, const DevPme& m, int step_off,
 }
 
 void launch_pme_energy(const DevPme& m, int n, double* out, cudaStream_t st) {
-    k_pme_energy_sum<<<1, 256, 0, st>>>(m, PME_CONV_CTAS, n, out);
+    k_pme_energy_sum<<<1, 256, 0, st>>>(m, PME_CONV_CTAS, (n + EXCL_NT - 1) / EXCL_NT, out);
 }
