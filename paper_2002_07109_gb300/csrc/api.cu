@@ -13,12 +13,15 @@
 #include "common.cuh"
 
 void nlist_set_smem_limit(size_t bytes);
-int diff_param_count();
+size_t diff_scratch(int n);
+int diff_sum_count();
 void launch_pair_forward(const DevSys& s, const Params& p, const float* qt, const float* sig, const float* eps, int T,
-                         int cur, double* F, double* eatom, double* esum, cudaStream_t st);
-void launch_pair_backward(const DevSys& s, const Params& p, const float* qt, const float* sig, const float* eps, int T,
-                          int cur, const double* U, double w, double* gpos, double* part, double* psum,
-                          cudaStream_t st);
+                         int cur, double* F, double* ecta, double* esum, cudaStream_t st);
+const double* launch_pair_backward(const DevSys& s, const Params& p, const float* qt, const float* sig, const float* eps,
+                                   int T, int cur, const double* U, double w, double* gpos, double* scratch,
+                                   cudaStream_t st);
+void diff_chain(const double* sums, const float* qt, const float* sig, const float* eps, int T, double* gq, double* gs,
+                double* ge);
 void launch_pair_hist(const DevSys& s, const Params& p, int cur, int ta, int tb, double r_max, int n_bins,
                       unsigned long long* hist, cudaStream_t st);
 void launch_msd(const DevSys& s, const double* rx, const double* ry, const double* rz, int cur, int t,
@@ -75,7 +78,7 @@ struct bounce_ctx {
     bool rows_valid = false;             // rows were requested for this topology and replica layout
     bool has_pme = false;
     DevPme pme{};
-    double* diff_part = nullptr;   // [NPAR n + NPAR] parameter partials and sums of the pair backward
+    double* diff_part = nullptr;   // scratch of the pair backward (diff_scratch)
     double e_self = 0.0;
     // cluster-pair path: allocated capacities (buffers grow, never shrink)
     int cl_cap_ncol = 0, cl_cap_ncl = 0, cl_cap_items = 0;
@@ -1954,24 +1957,24 @@ int bounce_pair_backward(bounce_ctx* c, int32_t T, const double* qt, const doubl
     if (r) return r;
     cudaSetDevice(c->cfg.device);
     cudaStream_t st = (cudaStream_t)stream;
-    const int np = diff_param_count();
-    if (!c->diff_part && (r = dalloc(c, &c->diff_part, (size_t)np * c->n + np))) return r;
+    if (!c->diff_part && (r = dalloc(c, &c->diff_part, diff_scratch(c->n)))) return r;
     const int cur = (int)(c->cur_step & 1);
-    double* psum = c->diff_part + (size_t)np * c->n;
-    launch_pair_backward(c->ds, c->pp, fq, fs, fe, T, cur, grad_forces, grad_energy, grad_pos, c->diff_part, psum, st);
-    std::vector<double> ps(np);
-    CU(cudaMemcpyAsync(ps.data(), psum, np * sizeof(double), cudaMemcpyDeviceToHost, st));
-    CU(cudaStreamSynchronize(st));
+    const double* sums =
+        launch_pair_backward(c->ds, c->pp, fq, fs, fe, T, cur, grad_forces, grad_energy, grad_pos, c->diff_part, st);
+    CU(cudaMemcpyAsync(c->h_out, sums, diff_sum_count() * sizeof(double), cudaMemcpyDeviceToHost, st));
+    r = check_err(c, st);
     const int M = BOUNCE_MAXT;
+    double gq[BOUNCE_MAXT], gs[BOUNCE_MAXT * BOUNCE_MAXT], ge[BOUNCE_MAXT * BOUNCE_MAXT];
+    diff_chain(c->h_out, fq, fs, fe, T, gq, gs, ge);
     for (int a = 0; a < T; ++a) {
-        if (grad_qt) grad_qt[a] = ps[a];
+        if (grad_qt) grad_qt[a] = gq[a];
         for (int b = 0; b < T; ++b) {
-            const int lo = std::min(a, b), hi = std::max(a, b);
-            if (grad_sig) grad_sig[a * T + b] = ps[M + lo * M + hi];
-            if (grad_eps) grad_eps[a * T + b] = ps[M + M * M + lo * M + hi];
+            const int k = std::min(a, b) * M + std::max(a, b);
+            if (grad_sig) grad_sig[a * T + b] = gs[k];
+            if (grad_eps) grad_eps[a * T + b] = ge[k];
         }
     }
-    return check_err(c, st);
+    return r;
 }
 
 const char* bounce_last_error(const bounce_ctx* c) {
