@@ -1207,9 +1207,7 @@ int bounce_set_topology(bounce_ctx* c, int32_t n, const int32_t* type, const dou
         (r = dalloc(c, &s.nlong, n)) || (r = dalloc(c, &s.rows, (size_t)n * s.cap)) ||
         (r = dalloc(c, &s.nseg, (size_t)n * BOUNCE_MAXT)) || (r = dalloc(c, &s.nshort, n)) || (r = dalloc(c, &s.srows, distinct_short ? (size_t)n * s.caps : 1)) ||
         (r = dalloc(c, &s.refx, n)) || (r = dalloc(c, &s.refy, n)) || (r = dalloc(c, &s.refz, n)) ||
-        (r = dalloc(c, &s.cell_atoms, n)) || (r = dalloc(c, &s.cell_phi, n)) || (r = dalloc(c, &s.cell_mol, n)) ||
-        (r = dalloc(c, &s.g0, n)) ||
-        (r = dalloc(c, &s.cell_type, n)) ||
+        (r = dalloc(c, &s.cell_phi, n)) || (r = dalloc(c, &s.cell_mt, n)) || (r = dalloc(c, &s.g0, n)) ||
         (r = dalloc(c, &s.done_ctr, 2)) ||
         (r = dalloc(c, &s.rebuild, 1)) || (r = dalloc(c, &s.err, 1)) ||
         (r = dalloc(c, &s.cnt, CNT_N)) || (r = dalloc(c, &c->d_step, 1)) || (r = dalloc(c, &c->terms, 6 * (size_t)n + 2048)) ||

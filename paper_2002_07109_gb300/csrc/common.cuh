@@ -137,12 +137,10 @@ struct DevSys {
     int* cell_count;
     int* cell_start;
     int* cell_fill;
-    int* cell_atoms;
-    float4* cell_phi;  // high position parts in cell order (coalesced candidate reads)
+    float4* cell_phi;  // high position parts in cell order (coalesced candidate reads); w = index (int bits)
     float4* g0;        // pair-sum gradient of each atom from k_pairs (x, y, z; w = row entries, int bits)
     unsigned int* done_ctr;  // [2] finished-CTA counters of the rebuild kernels (zero between launches)
-    int* cell_mol;     // molecule ids in cell order
-    int* cell_type;    // atom types in cell order
+    int2* cell_mt;     // molecule ids and atom types in cell order
     int ncx, ncy, ncz;
     float ox, oy, oz;        // grid origin (droplets)
     float ihx, ihy, ihz;     // inverse cell edges
