@@ -269,25 +269,49 @@ __device__ __forceinline__ void shift_split(float& h, float& l, float sh, float 
     l = (l - sl) + err;
 }
 
-// 4. neighbour lists (warp per cluster I): every atom j of a cluster
+// 4. neighbour lists (CTA per cluster I): every atom j of a cluster
 // J >= I of the columns in reach whose distance to I's bounding box (minimum
 // image per axis) is below the search radius, in a fixed order, as its slot
 // with the periodic image of the pair (or the per-pair code when the pair's
 // separation could reach half a box edge).  Every unordered pair of atoms
 // inside the cutoff then appears once: in the list of the lower cluster, and
 // for two atoms of one cluster with the lower slot as i.
-__global__ void __launch_bounds__(256) k_cl_search(DevSys s, Params p, int step_off, int force) {
+//
+// Bounded by the chain of one cluster (columns, boxes, atoms, each load
+// waiting for the last), so the chain is kept short: the columns in reach are
+// one prefix sum over the CTA's threads, the box tests run 128 clusters at a
+// time over the columns' concatenation, those that pass queue up in a ring,
+// and the atom tests take 64 queued clusters at a time, four loads in flight
+// per thread.  Votes and counts of the warps, exchanged once per step, keep
+// every entry in the order of (row, column, cluster, atom).  A warp per
+// cluster that walked the columns one by one (six clusters of 32 lanes) took
+// 97 us for 12,288 atoms, 120 us for 27,783 and 285 us for 98,304; this takes 31,
+// 50 and 170.
+constexpr int NB_NT = 128, NB_W = NB_NT / 32;  // threads and warps of a search or prune CTA
+constexpr int NB_PASS = 4;                     // atoms (entries) in flight per thread
+constexpr int NB_QUEUE = NB_PASS * NB_NT / CL;  // clusters of an atom-level step
+constexpr int NB_RING = 256;                   // queued clusters: < NB_QUEUE left over + 128 new
+
+__global__ void __launch_bounds__(NB_NT, 8) k_cl_search(DevSys s, Params p, int step_off, int force) {
     if (!cl_pending(s, force)) return;
+    __shared__ int run_start[NB_NT], run_off[NB_NT];  // non-empty columns: first candidate, first cluster less it
+    __shared__ int wsum[NB_W];
+    __shared__ int ring[NB_RING];
+    __shared__ int bcnt[2][NB_W];
+    __shared__ uint32_t acnt[2][NB_PASS * NB_W];
     const DevClu& c = s.cl;
-    const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, wl = tid >> 5;
     const int ncl = c.ncol * c.maxcl;
     const int cur = (int)((*s.step_base + step_off) & 1);
     const float Lx = p.Lhi[0], Ly = p.Lhi[1], Lz = p.Lhi[2];
+    const uint32_t below = (1u << lane) - 1u;
     bool overflow = false;
-    for (int I = blockIdx.x * wpb + (threadIdx.x >> 5); I < ncl; I += gridDim.x * wpb) {
-        const int col = I / c.maxcl, k = I - col * c.maxcl;
+    int bpar = 0, apar = 0;  // the count buffers alternate: one barrier per step
+    // the first clusters of all columns, then the second ones, ...: the unused slots of the columns come last
+    for (int t = blockIdx.x; t < ncl; t += gridDim.x) {
+        const int k = t / c.ncol, col = t - k * c.ncol, I = col * c.maxcl + k;
         if (k >= c.col_ncl[col]) {
-            if (lane == 0) {
+            if (tid == 0) {
                 c.lcnt[0][I] = 0;
                 c.lcnt[1][I] = 0;
             }
@@ -301,93 +325,166 @@ __global__ void __launch_bounds__(256) k_cl_search(DevSys s, Params p, int step_
         bool xall, yall;
         column_span(c.ncx, lo.x - R, hi.x + R, p.periodic ? 0.f : c.ox, c.ihx, p.periodic, xa, xb, xall);
         column_span(c.ncy, lo.y - R, hi.y + R, p.periodic ? 0.f : c.oy, c.ihy, p.periodic, ya, yb, yall);
-        int m0 = 0, m1 = 0;
-        const uint32_t below = (1u << lane) - 1u;
-        for (int yy = ya; yy <= yb; ++yy) {
-            const int cyn = p.periodic ? (yy % c.ncy + c.ncy) % c.ncy : yy;
-            for (int xx = xa; xx <= xb; ++xx) {
-                const int cxn = p.periodic ? (xx % c.ncx + c.ncx) % c.ncx : xx;
-                const int coln = cyn * c.ncx + cxn;
-                const int colb = coln * c.maxcl;
-                // the clusters J >= I of the column: all of them, or those after I in I's own column
-                const int nk = c.col_ncl[coln];
-                const int k0 = colb > I ? 0 : (colb == I - k ? k : nk);
-                for (int kb = k0; kb < nk; kb += 32) {
-                    // cluster level: boxes within the search radius (minimum image per axis)
-                    const int kk = kb + lane;
-                    bool near = false;
-                    if (kk < nk) {
-                        const float4 lj = c.bb_lo[colb + kk], hj = c.bb_hi[colb + kk];
-                        float dx = cx - 0.5f * (lj.x + hj.x), dy = cy - 0.5f * (lj.y + hj.y),
-                              dz = cz - 0.5f * (lj.z + hj.z);
-                        if (p.periodic) {
-                            dx -= rintf(dx * p.invL[0]) * Lx;
-                            dy -= rintf(dy * p.invL[1]) * Ly;
-                            dz -= rintf(dz * p.invL[2]) * Lz;
-                        }
-                        const float gx = fmaxf(fabsf(dx) - (ex + 0.5f * (hj.x - lj.x)), 0.f);
-                        const float gy = fmaxf(fabsf(dy) - (ey + 0.5f * (hj.y - lj.y)), 0.f);
-                        const float gz = fmaxf(fabsf(dz) - (ez + 0.5f * (hj.z - lj.z)), 0.f);
-                        near = gx * gx + gy * gy + gz * gz < c.rs2[0];
-                    }
-                    uint32_t qual = __ballot_sync(0xffffffffu, near);
-                    // atom level, four qualifying clusters per pass: lane = 8 q + t
-                    while (qual) {
-                        int pick = -1;
-                        uint32_t rest = qual;
-                        for (int q = 0; q <= (lane >> 3); ++q) {
-                            pick = rest ? __ffs(rest) - 1 : -1;
-                            rest = rest ? rest & (rest - 1) : 0u;
-                        }
-                        for (int q = 0; q < 4 && qual; ++q) qual &= qual - 1;
-                        const int sj = pick >= 0 ? (colb + kb + pick) * CL + (lane & 7) : 0;
-                        bool inL = false, inS = false;
-                        int code = NO_SHIFT;
-                        if (pick >= 0 && c.smol[sj] >= 0) {
-                            const float4 h = c.sphi[cur][sj];
-                            float dx = h.x - cx, dy = h.y - cy, dz = h.z - cz;
-                            if (p.periodic) {
-                                const int kx = (int)rintf(dx * p.invL[0]);
-                                const int ky = (int)rintf(dy * p.invL[1]);
-                                const int kz = (int)rintf(dz * p.invL[2]);
-                                dx -= kx * Lx;
-                                dy -= ky * Ly;
-                                dz -= kz * Lz;
-                                // image code of q_j - k L (the kernel subtracts k L from q_j)
-                                code = (kx + 1) * 9 + (ky + 1) * 3 + (kz + 1);
-                                if (fabsf(dx) + 2.f * ex >= 0.49f * Lx || fabsf(dy) + 2.f * ey >= 0.49f * Ly ||
-                                    fabsf(dz) + 2.f * ez >= 0.49f * Lz)
-                                    code = PER_PAIR;
-                            }
-                            const float gx = fmaxf(fabsf(dx) - ex, 0.f), gy = fmaxf(fabsf(dy) - ey, 0.f),
-                                        gz = fmaxf(fabsf(dz) - ez, 0.f);
-                            const float d2 = gx * gx + gy * gy + gz * gz;
-                            inL = d2 < c.rs2[0];
-                            inS = c.nlists > 1 && d2 < c.rs2[1];
-                        }
-                        const uint32_t bl = __ballot_sync(0xffffffffu, inL), bs = __ballot_sync(0xffffffffu, inS);
-                        const int ent = sj | (code << 27);
-                        if (inL) {
-                            const int pos = m0 + __popc(bl & below);
-                            if (pos < c.capj[0]) c.lst[0][(size_t)I * c.capj[0] + pos] = ent;
-                        }
-                        if (inS) {
-                            const int pos = m1 + __popc(bs & below);
-                            if (pos < c.capj[1]) c.lst[1][(size_t)I * c.capj[1] + pos] = ent;
-                        }
-                        m0 += __popc(bl);
-                        m1 += __popc(bs);
-                    }
+        const int nxs = xb - xa + 1, ncols = nxs * (yb - ya + 1);
+        int m0 = 0, m1 = 0;          // entries so far
+        int head = 0, tail = 0;      // ring: queued clusters
+        // atom level over up to 64 queued clusters: thread = 8 q + t of each pass
+        auto atoms = [&](int nq) {
+            int sj[NB_PASS], mj[NB_PASS];
+            float4 h[NB_PASS];
+#pragma unroll
+            for (int u = 0; u < NB_PASS; ++u) {
+                const int q = u * (NB_NT / CL) + (tid >> 3);
+                sj[u] = q < nq ? ring[(head + q) & (NB_RING - 1)] * CL + (tid & 7) : -1;
+                mj[u] = -1;
+                if (sj[u] >= 0) {
+                    mj[u] = c.smol[sj[u]];
+                    h[u] = c.sphi[cur][sj[u]];
                 }
             }
+            uint32_t bl[NB_PASS], bs[NB_PASS];
+#pragma unroll
+            for (int u = 0; u < NB_PASS; ++u) {
+                bool inL = false, inS = false;
+                int code = NO_SHIFT;
+                if (mj[u] >= 0) {
+                    float dx = h[u].x - cx, dy = h[u].y - cy, dz = h[u].z - cz;
+                    if (p.periodic) {
+                        const int kx = (int)rintf(dx * p.invL[0]);
+                        const int ky = (int)rintf(dy * p.invL[1]);
+                        const int kz = (int)rintf(dz * p.invL[2]);
+                        dx -= kx * Lx;
+                        dy -= ky * Ly;
+                        dz -= kz * Lz;
+                        // image code of q_j - k L (the kernel subtracts k L from q_j)
+                        code = (kx + 1) * 9 + (ky + 1) * 3 + (kz + 1);
+                        if (fabsf(dx) + 2.f * ex >= 0.49f * Lx || fabsf(dy) + 2.f * ey >= 0.49f * Ly ||
+                            fabsf(dz) + 2.f * ez >= 0.49f * Lz)
+                            code = PER_PAIR;
+                    }
+                    const float gx = fmaxf(fabsf(dx) - ex, 0.f), gy = fmaxf(fabsf(dy) - ey, 0.f),
+                                gz = fmaxf(fabsf(dz) - ez, 0.f);
+                    const float d2 = gx * gx + gy * gy + gz * gz;
+                    inL = d2 < c.rs2[0];
+                    inS = c.nlists > 1 && d2 < c.rs2[1];
+                }
+                bl[u] = __ballot_sync(0xffffffffu, inL);
+                bs[u] = __ballot_sync(0xffffffffu, inS);
+                sj[u] |= code << 27;
+                if (lane == 0) acnt[apar][u * NB_W + wl] = __popc(bl[u]) | __popc(bs[u]) << 16;
+            }
+            __syncthreads();
+            // entries of the passes and warps before, both lists packed
+            const uint32_t v = lane < NB_PASS * NB_W ? acnt[apar][lane] : 0u;
+            uint32_t x = v;
+#pragma unroll
+            for (int o = 1; o < NB_PASS * NB_W; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o) x += y;
+            }
+#pragma unroll
+            for (int u = 0; u < NB_PASS; ++u) {
+                const uint32_t before = __shfl_sync(0xffffffffu, x - v, u * NB_W + wl);
+                if (bl[u] >> lane & 1) {
+                    const int pos = m0 + (int)(before & 0xffffu) + __popc(bl[u] & below);
+                    if (pos < c.capj[0]) c.lst[0][(size_t)I * c.capj[0] + pos] = sj[u];
+                }
+                if (bs[u] >> lane & 1) {
+                    const int pos = m1 + (int)(before >> 16) + __popc(bs[u] & below);
+                    if (pos < c.capj[1]) c.lst[1][(size_t)I * c.capj[1] + pos] = sj[u];
+                }
+            }
+            const uint32_t all = __shfl_sync(0xffffffffu, x, NB_PASS * NB_W - 1);
+            m0 += all & 0xffffu;
+            m1 += all >> 16;
+            head += nq;
+            apar ^= 1;
+        };
+        for (int cb = 0; cb < ncols; cb += NB_NT) {
+            // the clusters J >= I of a column: all of them, or those from I on in I's own column
+            int off = 0, len = 0;
+            if (cb + tid < ncols) {
+                const int ry = (cb + tid) / nxs, yy = ya + ry, xx = xa + (cb + tid) - ry * nxs;
+                const int cyn = p.periodic ? (yy % c.ncy + c.ncy) % c.ncy : yy;
+                const int cxn = p.periodic ? (xx % c.ncx + c.ncx) % c.ncx : xx;
+                const int coln = cyn * c.ncx + cxn;
+                const int k0 = coln > col ? 0 : k;
+                len = coln >= col ? max(c.col_ncl[coln] - k0, 0) : 0;
+                off = coln * c.maxcl + k0;
+            }
+            // prefix over the columns: candidates (low 24 bits) and non-empty columns
+            const int v = len | (len > 0) << 24;
+            int x = v;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o) x += y;
+            }
+            __syncthreads();  // (the last batch's runs are read)
+            if (lane == 31) wsum[wl] = x;
+            __syncthreads();
+            int total = 0;
+#pragma unroll
+            for (int w = 0; w < NB_W; ++w) {
+                if (w == wl) x += total;
+                total += wsum[w];
+            }
+            x -= v;
+            if (len > 0) {
+                run_start[x >> 24] = x & 0xffffff;
+                run_off[x >> 24] = off - (x & 0xffffff);
+            }
+            const int nr = total >> 24, nt = total & 0xffffff;
+            __syncthreads();
+            int t0 = 0;
+            do {  // (once where no column has a cluster, for what is left in the ring)
+                // cluster level: boxes within the search radius (minimum image per axis)
+                const int tt = t0 + tid;
+                bool near = false;
+                int J = 0;
+                if (tt < nt) {
+                    int r = 0;  // last run with run_start <= tt
+#pragma unroll
+                    for (int st = NB_NT / 2; st > 0; st >>= 1)
+                        if (r + st < nr && run_start[r + st] <= tt) r += st;
+                    J = tt + run_off[r];
+                    const float4 lj = c.bb_lo[J], hj = c.bb_hi[J];
+                    float dx = cx - 0.5f * (lj.x + hj.x), dy = cy - 0.5f * (lj.y + hj.y),
+                          dz = cz - 0.5f * (lj.z + hj.z);
+                    if (p.periodic) {
+                        dx -= rintf(dx * p.invL[0]) * Lx;
+                        dy -= rintf(dy * p.invL[1]) * Ly;
+                        dz -= rintf(dz * p.invL[2]) * Lz;
+                    }
+                    const float gx = fmaxf(fabsf(dx) - (ex + 0.5f * (hj.x - lj.x)), 0.f);
+                    const float gy = fmaxf(fabsf(dy) - (ey + 0.5f * (hj.y - lj.y)), 0.f);
+                    const float gz = fmaxf(fabsf(dz) - (ez + 0.5f * (hj.z - lj.z)), 0.f);
+                    near = gx * gx + gy * gy + gz * gz < c.rs2[0];
+                }
+                const uint32_t bn = __ballot_sync(0xffffffffu, near);
+                if (lane == 0) bcnt[bpar][wl] = __popc(bn);
+                __syncthreads();
+                int at = tail;
+#pragma unroll
+                for (int w = 0; w < NB_W; ++w) {
+                    if (w == wl && near) ring[(at + __popc(bn & below)) & (NB_RING - 1)] = J;
+                    at += bcnt[bpar][w];
+                }
+                tail = at;
+                bpar ^= 1;
+                __syncthreads();
+                t0 += NB_NT;
+                const int least = cb + NB_NT >= ncols && t0 >= nt ? 1 : NB_QUEUE;
+                while (tail - head >= least) atoms(min(tail - head, NB_QUEUE));
+            } while (t0 < nt);
         }
-        if (lane == 0) {
+        if (tid == 0) {
             c.lcnt[0][I] = min(m0, c.capj[0]);
             c.lcnt[1][I] = c.nlists > 1 ? min(m1, c.capj[1]) : 0;
         }
         overflow = overflow || m0 > c.capj[0] || (c.nlists > 1 && m1 > c.capj[1]);
     }
-    if (overflow) atomicOr(s.err, BERR_LIST_OVERFLOW);
+    if (overflow && tid == 0) atomicOr(s.err, BERR_LIST_OVERFLOW);
     if (!cl_last_cta(&c.done_ctr[1])) return;
     if (threadIdx.x == 0) {
         *c.rebuild = 0;
@@ -431,48 +528,62 @@ __device__ __forceinline__ bool prune_keep(const DevSys& s, const Params& p, int
 // FP32 with a margin, so that no pair the exact test would keep is dropped),
 // in list order.  The step kernel raises the flag when an atom's slot copy has moved half the
 // prune skin since this launch, which it records here.
-__global__ void __launch_bounds__(256) k_cl_prune(DevSys s, Params p, int step_off, int force) {
+//
+// Bounded by the chain of one list (entries, their positions, the vote): four
+// passes of 32 entries are in flight per warp (two: 30 us for 12,288 atoms, 73 us
+// for 98,304; four: 26 and 67).  A CTA per cluster takes 24 and 98 us.
+__global__ void __launch_bounds__(NB_NT, 8) k_cl_prune(DevSys s, Params p, int step_off, int force) {
     chain_enter();
     if (!(force || *s.cl.prune)) return;
     const DevClu& c = s.cl;
-    const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5, wl = threadIdx.x >> 5;
-    __shared__ float4 s_hi[8][CL], s_lo[8][CL];
+    const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
+    __shared__ float4 s_hi[NB_W][CL], s_lo[NB_W][CL];
     const int ncl = c.ncol * c.maxcl;
     const int cur = (int)((*s.step_base + step_off) & 1);
     const uint32_t below = (1u << lane) - 1u;
-    for (int I = blockIdx.x * wpb + wl; I < ncl; I += gridDim.x * wpb) {
+    for (int t = blockIdx.x * NB_W + wl; t < ncl; t += gridDim.x * NB_W) {
+        const int kt = t / c.ncol, I = (t - kt * c.ncol) * c.maxcl + kt;  // the columns' unused slots come last
+        int n[2];
+        n[0] = c.lcnt[0][I];
+        n[1] = c.nlists > 1 ? c.lcnt[1][I] : 0;
         __syncwarp();
         if (lane < CL) {
             // padding slots (no atom) are placed out of reach: their copies in
             // the buffer the step kernel writes are never refreshed
             const bool real = c.smol[I * CL + lane] >= 0;
-            const float4 far = make_float4(1e30f, 1e30f, 1e30f, 0.f);
-            s_hi[wl][lane] = real ? c.sphi[cur][I * CL + lane] : far;
+            const float4 h = c.sphi[cur][I * CL + lane];
+            s_hi[wl][lane] = real ? h : make_float4(1e30f, 1e30f, 1e30f, 0.f);
             s_lo[wl][lane] = real ? c.splo[cur][I * CL + lane] : make_float4(0.f, 0.f, 0.f, 0.f);
-            c.pref[I * CL + lane] = c.sphi[cur][I * CL + lane];
+            c.pref[I * CL + lane] = h;
         }
         __syncwarp();
-        for (int L = 0; L < c.nlists; ++L) {
-            const int n = c.lcnt[L][I];
+#pragma unroll
+        for (int L = 0; L < 2; ++L) {
+            if (L >= c.nlists) break;
             const int* src = c.lst[L] + (size_t)I * c.capj[L];
             int* dst = c.plst[L] + (size_t)I * c.capj[L];
             int m = 0;
             const float R2 = c.prs2[L];
-            // two passes of 32 entries per iteration: their loads are in flight together
-            for (int e0 = 0; e0 < n; e0 += 64) {
+            for (int e0 = 0; e0 < n[L]; e0 += 32 * NB_PASS) {
+                int ent[NB_PASS];
+                float4 h[NB_PASS];
                 // (an entry's image code fills its top bits: validity comes from the index)
-                const int ea = e0 + lane, eb = ea + 32;
-                const bool va = ea < n, vb = eb < n;
-                const int enta = va ? src[ea] : 0, entb = vb ? src[eb] : 0;
-                const float4 ha = va ? c.sphi[cur][enta & 0x07FFFFFF] : make_float4(0.f, 0.f, 0.f, 0.f);
-                const float4 hb = vb ? c.sphi[cur][entb & 0x07FFFFFF] : make_float4(0.f, 0.f, 0.f, 0.f);
-                const bool ka = va && prune_keep(s, p, cur, enta, ha, s_hi[wl], s_lo[wl], R2);
-                const bool kb = vb && prune_keep(s, p, cur, entb, hb, s_hi[wl], s_lo[wl], R2);
-                const uint32_t ba = __ballot_sync(0xffffffffu, ka), bb = __ballot_sync(0xffffffffu, kb);
-                if (ka) dst[m + __popc(ba & below)] = enta;
-                m += __popc(ba);
-                if (kb) dst[m + __popc(bb & below)] = entb;
-                m += __popc(bb);
+#pragma unroll
+                for (int u = 0; u < NB_PASS; ++u) {
+                    const int e = e0 + 32 * u + lane;
+                    ent[u] = e < n[L] ? src[e] : 0;
+                }
+#pragma unroll
+                for (int u = 0; u < NB_PASS; ++u)
+                    h[u] = e0 + 32 * u + lane < n[L] ? c.sphi[cur][ent[u] & 0x07FFFFFF] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int u = 0; u < NB_PASS; ++u) {
+                    const bool keep =
+                        e0 + 32 * u + lane < n[L] && prune_keep(s, p, cur, ent[u], h[u], s_hi[wl], s_lo[wl], R2);
+                    const uint32_t b = __ballot_sync(0xffffffffu, keep);
+                    if (keep) dst[m + __popc(b & below)] = ent[u];
+                    m += __popc(b);
+                }
             }
             if (lane == 0) {
                 c.pcnt[L][I] = m;
@@ -689,8 +800,8 @@ void launch_cluster_rebuild(const DevSys& s, const Params& p, int step_off, bool
     launch_chained(k_cl_scatter, gb, tb, 0, st, s, p, step_off, f);
     launch_chained(k_cl_sort, std::min(s.cl.ncol, 152 * 8), SORT_NT, 0, st, s, p, step_off, f);
     const int ncl = s.cl.ncol * s.cl.maxcl;
-    launch_chained(k_cl_search, std::min((ncl + 7) / 8, 152 * 8), 256, 0, st, s, p, step_off, f);
-    launch_chained(k_cl_prune, std::min((ncl + 7) / 8, 152 * 8), 256, 0, st, s, p, step_off, f);
+    launch_chained(k_cl_search, std::min(ncl, 152 * 8), NB_NT, 0, st, s, p, step_off, f);
+    launch_chained(k_cl_prune, std::min((ncl + NB_W - 1) / NB_W, 152 * 8), NB_NT, 0, st, s, p, step_off, f);
 }
 
 // CTAs of a pair kernel that fit on the GPU at once (the warps fetch their
