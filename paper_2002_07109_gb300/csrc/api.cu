@@ -460,6 +460,7 @@ void fill_params(bounce_ctx* c, const std::vector<double>& sig, const std::vecto
     p.dt_half_f = (float)(0.5 * p.dt);
     p.c1 = std::exp(-g.gamma_per_fs * g.dt_fs);
     p.skin_half2 = std::isfinite(rl) ? 0.25 * g.skin * g.skin : INFINITY;
+    p.skin_half2f = (float)p.skin_half2;
     p.key0 = (uint32_t)(g.seed & 0xFFFFFFFFull);
     p.key1 = (uint32_t)(g.seed >> 32);
 }
@@ -659,6 +660,7 @@ int setup_clusters(bounce_ctx* c, const double* q, const HostBox& hb) {
         nk.rs2[L] = (float)(rm * rm);
     }
     nk.cskin_half2 = 0.25 * cskin * cskin;
+    nk.cskin_half2f = (float)nk.cskin_half2;
     nk.capitems = ncl * (nk.capj[0] / BOUNCE_CL_EPW + 1);
     // pruned lists: entries within r + dp of some atom of I, dp = half the
     // cluster skin up to CL_PRUNE_SKIN (10 mA margin for the FP32 test),

@@ -52,6 +52,7 @@ struct DevClu {
     float rs2[2];            // squared search radii of the lists (with margins)
     float rsx[2];            // the radii themselves
     double cskin_half2;      // rebuild when an atom moved more than skin/2 since the build
+    float cskin_half2f;      // the same in FP32 (moved_beyond)
     int* col_count;          // [ncol]
     int* col_start;          // [ncol + 1]
     int* col_fill;           // [ncol]
@@ -223,6 +224,7 @@ struct Params {
     float beta_f, dt_half_f;     // beta and dt / 2 in FP32 (the jump step's bound of the Poisson mean)
     double c1;
     double skin_half2;
+    float skin_half2f;           // the same in FP32 (moved_beyond)
     uint32_t key0, key1;
 };
 
@@ -318,13 +320,83 @@ __device__ __forceinline__ int poisson_invert_f32(float u, float mu_c) {
     return k;
 }
 
+// Conversions between FP64, FP32 and the fixed-point sums on the integer pipes.
+// A warp's FP64 instruction, the conversions F2F and I2F of 64 bits among them,
+// holds this GPU's FP64 pipe for ~16 SM cycles, an integer one for a quarter of
+// a cycle; two thirds of the step kernels' FP64 work were conversions.  Each of
+// these returns the bits of the instruction that it stands for.
+
+// (double)f.
+__device__ __forceinline__ double widen(float f) {
+    const bool small = fabsf(f) < 1.17549435e-38f;  // subnormals and zero
+    const uint32_t u = __float_as_uint(small ? f * 18446744073709551616.f : f), a = u & 0x7fffffffu;
+    uint32_t hi = (a >> 3) + (small ? 0x34000000u : 0x38000000u);  // exponent bias 1023 - 127, less the 2^64
+    if (a >= 0x7f800000u) hi |= 0x7ff00000u;                       // infinity and NaN
+    if (a == 0u) hi = 0u;
+    return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)(u << 29));
+}
+
+// The FP32 value nearest to x (ties to even) of an x whose exponent lies in
+// that of normal FP32 values; h is the high word without the sign.
+__device__ __forceinline__ float narrow_normal(double x, uint32_t h, bool& up) {
+    const uint32_t lo = (uint32_t)__double2loint(x), t = (h - 0x38000000u) << 3 | lo >> 29, r = lo << 3;
+    up = r > 0x80000000u || (r == 0x80000000u && (t & 1u));
+    return __uint_as_float((t + (up ? 1u : 0u)) | ((uint32_t)__double2hiint(x) & 0x80000000u));
+}
+
+// (float)x.
+__device__ __forceinline__ float narrow(double x) {
+    const uint32_t h = (uint32_t)__double2hiint(x) & 0x7fffffffu;
+    if (h - 0x38100000u >= 0x0fe00000u) return __double2float_rn(x);  // outside 2^-126 .. 2^128
+    bool up;
+    return narrow_normal(x, h, up);
+}
+
+// hi = (float)x and lo = (float)(x - hi): the rest is the low 29 bits of the
+// significand, less 2^29 where hi was rounded away from zero.
+__device__ __forceinline__ void split_double(double x, float& hi, float& lo) {
+    const uint32_t h = (uint32_t)__double2hiint(x) & 0x7fffffffu;
+    if (h - 0x3b600000u >= 0x0c800000u) {  // outside 2^-73 .. 2^127: the rest might be subnormal
+        hi = __double2float_rn(x);
+        lo = __double2float_rn(x - (double)hi);
+        return;
+    }
+    bool up;
+    hi = narrow_normal(x, h, up);
+    int rest = (int)((uint32_t)__double2loint(x) & 0x1fffffffu) - (up ? 0x20000000 : 0);
+    if (__double2hiint(x) < 0) rest = -rest;
+    // times 2^(e - 52), e = (h >> 20) - 1023
+    lo = (float)rest * __uint_as_float(((h >> 20) - 1075u + 127u) << 23);
+}
+
+// (float)((double)a 2^-32) for |a| < 2^53, where the conversion to FP64 is
+// exact (2e6 kcal/mol/A; beyond, one rounding instead of two): the 32 leading
+// bits with the rest folded into the lowest of them round as the whole does.
+__device__ __forceinline__ float unfix32(long long a) {
+    const unsigned long long m = a < 0 ? 0ull - (unsigned long long)a : (unsigned long long)a;
+    const int lz = __clzll((long long)m);
+    if (lz == 64) return 0.f;
+    const unsigned long long n = m << lz;
+    const float f = __uint2float_rn((uint32_t)(n >> 32) | ((uint32_t)n ? 1u : 0u)) * __uint_as_float((uint32_t)(127 - lz) << 23);
+    return a < 0 ? -f : f;
+}
+
+// x x + y y + z z > lim, settled in FP32 unless the two are within 2e-6 of
+// each other (FP32 errors stay below 5e-7).
+__device__ __forceinline__ bool moved_beyond(double x, double y, double z, double lim, float limf) {
+    const float fx = narrow(x), fy = narrow(y), fz = narrow(z), d = fx * fx + fy * fy + fz * fz;
+    if (!(d > limf * 0.999998f)) return false;
+    return d > limf * 1.000002f || x * x + y * y + z * z > lim;
+}
+
 // x wrapped into [0, L): the multiple of L from the product with 1/L (no
 // FP64 division on the per-step path), moved by one where the product's
-// rounding put x on the wrong side of a multiple.
+// rounding put x on the wrong side of a multiple (compared as integers: the
+// bits of non-negative doubles have the order of their values).
 __device__ __forceinline__ double wrap_box(double x, double L, double iL) {
     double w = x - L * floor(x * iL);
-    if (w < 0.0) w += L;
-    else if (w >= L) w -= L;
+    if (__double2hiint(w) < 0) w += L;
+    else if (__double_as_longlong(w) >= __double_as_longlong(L)) w -= L;
     return w;
 }
 

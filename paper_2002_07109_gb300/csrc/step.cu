@@ -65,16 +65,15 @@ struct JumpSmem {
     unsigned long long cnt[3];    // proposals, accepts, near ties
 };
 
-// Split FP32 copy (hi, lo) of the position x - of: the slot copies of the
-// cluster lists keep the image of the last build (continuous motion across
-// faces), whatever the wrap of phi.
-__device__ __forceinline__ void split_pos(double x, double y, double z, double ox, double oy, double oz, float w_hi,
-                                          float w_lo, float4& ph, float4& pl) {
-    const double a = x - ox, b = y - oy, c = z - oz;
-    const float hx = __double2float_rn(a), hy = __double2float_rn(b), hz = __double2float_rn(c);
-    ph = make_float4(hx, hy, hz, w_hi);
-    pl = make_float4(__double2float_rn(a - (double)hx), __double2float_rn(b - (double)hy),
-                     __double2float_rn(c - (double)hz), w_lo);
+// Split FP32 copy (hi, lo) of a position.  (For the slot copies of the cluster
+// lists the caller subtracts the atom's image offset of the last build:
+// continuous motion across faces, whatever the wrap of phi.)
+__device__ __forceinline__ void split_pos(double x, double y, double z, float w_hi, float w_lo, float4& ph, float4& pl) {
+    split_double(x, ph.x, pl.x);
+    split_double(y, ph.y, pl.y);
+    split_double(z, ph.z, pl.z);
+    ph.w = w_hi;
+    pl.w = w_lo;
 }
 
 // Lane-parallel (warp 0): quantities of the jump step of atom `a` that need FP64.
@@ -91,7 +90,7 @@ __device__ __forceinline__ void jump_prep(const DevSys& s, const Params& p, Jump
         for (int b = 0; b < BOUNCE_MAXT; ++b) {
             const double lt = p.lt_d[t * BOUNCE_MAXT + b];
             W += (uint32_t)s.nseg[(size_t)i * BOUNCE_MAXT + b] * p.lq[t * BOUNCE_MAXT + b];
-            js.slt[a][b] = __double2float_rn(__dmul_rn(sp, lt));
+            js.slt[a][b] = narrow(__dmul_rn(sp, lt));
         }
         n = __dmul_rn((double)W, 1.52587890625e-05);
     } else {
@@ -106,14 +105,14 @@ __device__ __forceinline__ void jump_prep(const DevSys& s, const Params& p, Jump
     float muc = 0.f;
     if (mu > 0.0) {
         nch = (int)ceil(__dmul_rn(mu, 0.0625));  // mu / 16, exact
-        muc = __double2float_rn(nch == 1 ? mu : __ddiv_rn(mu, (double)nch));
+        muc = narrow(nch == 1 ? mu : __ddiv_rn(mu, (double)nch));
     }
     js.s[a] = sp;
-    js.sl[a] = __double2float_rn(__dmul_rn(sp, Ls));
+    js.sl[a] = narrow(__dmul_rn(sp, Ls));
     if (!p.typed) js.slt[a][0] = js.sl[a];
-    js.vf[a][0] = __double2float_rn(vx);
-    js.vf[a][1] = __double2float_rn(vy);
-    js.vf[a][2] = __double2float_rn(vz);
+    js.vf[a][0] = narrow(vx);
+    js.vf[a][1] = narrow(vy);
+    js.vf[a][2] = narrow(vz);
     js.muc[a] = muc;
     js.nch[a] = nch;
 }
@@ -597,9 +596,8 @@ __global__ void __launch_bounds__(NW * 32, 3) k_step(DevSys s, Params p, int var
             sSlot[a] = sl;
             const size_t ns = s.cl.on ? (size_t)s.cl.ncol * s.cl.maxcl * BOUNCE_CL : (size_t)s.n;
             unsigned long long* acc = s.cl.on ? s.cl.acc : s.tl.acc;
-            g = make_float4((float)((double)(long long)acc[sl] * CL_UNFIX),
-                            (float)((double)(long long)acc[ns + sl] * CL_UNFIX),
-                            (float)((double)(long long)acc[2 * ns + sl] * CL_UNFIX), 0.f);
+            g = make_float4(unfix32((long long)acc[sl]), unfix32((long long)acc[ns + sl]),
+                            unfix32((long long)acc[2 * ns + sl]), 0.f);
             acc[sl] = 0ull;
             acc[ns + sl] = 0ull;
             acc[2 * ns + sl] = 0ull;
@@ -683,14 +681,14 @@ __global__ void __launch_bounds__(NW * 32, 3) k_step(DevSys s, Params p, int var
         const int i = base + lane;
         double vx = sV[lane][0], vy = sV[lane][1], vz = sV[lane][2];
         if (do_j2) {
-            vx += (double)js.dv[lane][0];
-            vy += (double)js.dv[lane][1];
-            vz += (double)js.dv[lane][2];
+            vx += widen(js.dv[lane][0]);
+            vy += widen(js.dv[lane][1]);
+            vz += widen(js.dv[lane][2]);
         }
         const double c = hk * sKick[lane];
-        vx -= c * (double)sG[lane][0];
-        vy -= c * (double)sG[lane][1];
-        vz -= c * (double)sG[lane][2];
+        vx -= c * widen(sG[lane][0]);
+        vy -= c * widen(sG[lane][1]);
+        vz -= c * widen(sG[lane][2]);
         if (hr != 0.0) {
             const double cr = hr * sKick[lane];
             vx -= cr * s.grecip[i];
@@ -699,9 +697,9 @@ __global__ void __launch_bounds__(NW * 32, 3) k_step(DevSys s, Params p, int var
         }
         if (ext && hout != 0.0) {
             const double co = hout * sKick[lane];
-            vx -= co * (double)sGp[lane][0];
-            vy -= co * (double)sGp[lane][1];
-            vz -= co * (double)sGp[lane][2];
+            vx -= co * widen(sGp[lane][0]);
+            vy -= co * widen(sGp[lane][1]);
+            vz -= co * widen(sGp[lane][2]);
         }
         sV[lane][0] = vx;
         sV[lane][1] = vy;
@@ -717,18 +715,18 @@ __global__ void __launch_bounds__(NW * 32, 3) k_step(DevSys s, Params p, int var
         const int i = base + lane;
         double vx = sV[lane][0], vy = sV[lane][1], vz = sV[lane][2];
         if (do_j1) {
-            vx += (double)js.dv[lane][0];
-            vy += (double)js.dv[lane][1];
-            vz += (double)js.dv[lane][2];
+            vx += widen(js.dv[lane][0]);
+            vy += widen(js.dv[lane][1]);
+            vz += widen(js.dv[lane][2]);
         }
         if (do_aoa) {
             const double h = 0.5 * p.dt;
             double x = sQ[lane][0] + h * vx, y = sQ[lane][1] + h * vy, z = sQ[lane][2] + h * vz;
             // O: the Box-Muller normals drawn ahead (Philox slot 0, stream 0)
             const double sd = sOsd[lane];
-            vx = p.c1 * vx + sd * (double)sNz[lane][0];
-            vy = p.c1 * vy + sd * (double)sNz[lane][1];
-            vz = p.c1 * vz + sd * (double)sNz[lane][2];
+            vx = p.c1 * vx + sd * widen(sNz[lane][0]);
+            vy = p.c1 * vy + sd * widen(sNz[lane][1]);
+            vz = p.c1 * vz + sd * widen(sNz[lane][2]);
             x += h * vx;
             y += h * vy;
             z += h * vz;
@@ -741,26 +739,24 @@ __global__ void __launch_bounds__(NW * 32, 3) k_step(DevSys s, Params p, int var
                 wy = wrap_box(y, p.Ld[1], p.iLd[1]);
                 wz = wrap_box(z, p.Ld[2], p.iLd[2]);
             }
-            const float hx = __double2float_rn(wx), hy = __double2float_rn(wy), hz = __double2float_rn(wz);
-            const float4 ph = make_float4(hx, hy, hz, sHw[lane]);
-            const float4 pl = make_float4(__double2float_rn(wx - (double)hx), __double2float_rn(wy - (double)hy),
-                                          __double2float_rn(wz - (double)hz), sLw[lane]);
+            float4 ph, pl;
+            split_pos(wx, wy, wz, sHw[lane], sLw[lane], ph, pl);
             s.phi[nxt][i] = ph;
             s.plo[nxt][i] = pl;
             const double ex = x - sRef[lane][0], ey = y - sRef[lane][1], ez = z - sRef[lane][2];
             if (s.rows_flag && ((s.rows_move >> __float_as_int(sLw[lane])) & 1) &&
-                ex * ex + ey * ey + ez * ez > p.skin_half2)
+                moved_beyond(ex, ey, ez, p.skin_half2, p.skin_half2f))
                 atomicOr(s.rebuild, 1);
             if (s.cl.on) {
                 // slot-ordered copy for the cluster pair kernel (in the image of the
                 // build); displacement since the cluster build
                 const int sl = sSlot[lane];
                 float4 ch = ph, cw = pl;
-                if (p.periodic) split_pos(x, y, z, s.cl.cofx[i], s.cl.cofy[i], s.cl.cofz[i], ph.w, pl.w, ch, cw);
+                if (p.periodic) split_pos(x - s.cl.cofx[i], y - s.cl.cofy[i], z - s.cl.cofz[i], ph.w, pl.w, ch, cw);
                 s.cl.sphi[nxt][sl] = ch;
                 s.cl.splo[nxt][sl] = cw;
                 const double cx = x - sCref[lane][0], cy = y - sCref[lane][1], cz = z - sCref[lane][2];
-                if (cx * cx + cy * cy + cz * cz > s.cl.cskin_half2) atomicOr(s.cl.rebuild, 1);
+                if (moved_beyond(cx, cy, cz, s.cl.cskin_half2, s.cl.cskin_half2f)) atomicOr(s.cl.rebuild, 1);
                 // displacement since the last prune of the lists
                 const float4 pr = s.cl.pref[sl];
                 const float px = ch.x - pr.x, py = ch.y - pr.y, pz = ch.z - pr.z;
@@ -807,7 +803,7 @@ __device__ __forceinline__ void jump_thread(const DevSys& s, const Params& p, in
         // Poisson draw settle M = 0 without the FP64 set-up: expneg_f32 is
         // within 1e-6 of exp(-x), so u <= expneg_f32(mu_f) (1 - 4e-6) implies
         // u <= expneg_f32(float(mu)), which is the exact path's M = 0.
-        const float fx = __double2float_rn(vx), fy = __double2float_rn(vy), fz = __double2float_rn(vz);
+        const float fx = narrow(vx), fy = narrow(vy), fz = narrow(vz);
         const float spf = sqrtf(fx * fx + fy * fy + fz * fz);
         const float muf = p.beta_f * spf * p.Lstar_f[ti] * (float)s.nlong[i] * p.dt_half_f * 1.00001f;
         if (muf < 1.f) {
@@ -830,7 +826,7 @@ __device__ __forceinline__ void jump_thread(const DevSys& s, const Params& p, in
             ast[b] = st;
             W += (uint32_t)nb * p.lq[ti * BOUNCE_MAXT + b];
             st += nb;
-            slt[b] = __double2float_rn(__dmul_rn(sp, p.lt_d[ti * BOUNCE_MAXT + b]));
+            slt[b] = narrow(__dmul_rn(sp, p.lt_d[ti * BOUNCE_MAXT + b]));
         }
         acum[BOUNCE_MAXT] = W;
         n = __dmul_rn((double)W, 1.52587890625e-05);
@@ -844,7 +840,7 @@ __device__ __forceinline__ void jump_thread(const DevSys& s, const Params& p, in
     }
     if (!(mu > 0.0)) return;
     const int nch = (int)ceil(__dmul_rn(mu, 0.0625));
-    const float muc = __double2float_rn(nch == 1 ? mu : __ddiv_rn(mu, (double)nch));
+    const float muc = narrow(nch == 1 ? mu : __ddiv_rn(mu, (double)nch));
     int M = 0;
     for (int c = 0; c < nch; ++c) {
         const float u = u24(rng_atom(s, p, BOUNCE_POISSON_SLOT | (uint32_t)c, i, step, stream).x);
@@ -862,10 +858,10 @@ __device__ __forceinline__ void jump_thread(const DevSys& s, const Params& p, in
     }
     nprop += M;
     if (M == 0) return;
-    const float sl = __double2float_rn(__dmul_rn(sp, Ls));
+    const float sl = narrow(__dmul_rn(sp, Ls));
     if (!p.typed) slt[0] = sl;
-    const float sp_f = __double2float_rn(sp);
-    float fvx = __double2float_rn(vx), fvy = __double2float_rn(vy), fvz = __double2float_rn(vz);
+    const float sp_f = narrow(sp);
+    float fvx = narrow(vx), fvy = narrow(vy), fvz = narrow(vz);
     const int* row = s.rows + (size_t)i * s.cap;
     const int an = s.nlong[i];
     for (int k = 1; k <= M; ++k) {
@@ -939,21 +935,27 @@ __device__ __forceinline__ void jump_lite(const DevSys& s, const Params& p, int 
                                           double& vz, int& nprop, int& nacc, int& near) {
     float dx, dy, dz;
     jump_thread(s, p, cur, i, type_of(alo), vx, vy, vz, step, stream, ahi, alo, dx, dy, dz, nprop, nacc, near);
-    vx += (double)dx;
-    vy += (double)dy;
-    vz += (double)dz;
+    if (dx != 0.f || dy != 0.f || dz != 0.f) {  // (rare)
+        vx += widen(dx);
+        vy += widen(dy);
+        vz += widen(dz);
+    }
 }
 
-// Resident CTAs per SM the thread-per-atom kernel is compiled for: three
-// fit the 98,304-atom box's 384 CTAs in one wave (the register cap costs a
-// few spills around the jump phases, less than a second wave).
-#ifndef LITE_MIN_CTAS
-#define LITE_MIN_CTAS 3
-#endif
+// Threads of a thread-per-atom CTA, and CTAs per SM it is compiled for.  The
+// kernel is bound by the latency of its loads and by FP64 work (~40 FP64
+// instructions a warp, each ~16 SM cycles; 110 before the conversions went to
+// the integer pipes), so that CTAs of two warps, which spread the atoms evenly
+// over the SMs, are best: 12,288 atoms took 48 CTAs of eight warps, two SMs of
+// three idle.  Up to eight CTAs an SM keep every value in registers; twelve
+// fit the 98,304-atom box into one wave for a few spills around the jump
+// phases.  24.5 -> 13 us a step of 12,288 atoms, 41 -> 28 us of 98,304.
+constexpr int LITE_T = 64, LITE_FEW = 8, LITE_MANY = 12;
 
-template <int BOUNCE>
-__global__ void __launch_bounds__(256, LITE_MIN_CTAS) k_step_lite(DevSys s, Params p, int variant, int step_off,
-                                                                  double hr, int ext, double hout) {
+template <int BOUNCE, int CTAS>
+__global__ void __launch_bounds__(LITE_T, CTAS) k_step_lite(const __grid_constant__ DevSys s,
+                                                                   const __grid_constant__ Params p, int variant,
+                                                                   int step_off, double hr, int ext, double hout) {
     __shared__ unsigned long long cnt[4];
     chain_enter();
     if (threadIdx.x < 4) cnt[threadIdx.x] = 0ull;
@@ -973,17 +975,15 @@ __global__ void __launch_bounds__(256, LITE_MIN_CTAS) k_step_lite(DevSys s, Para
     int sl = i;
     float4 ahi = make_float4(0.f, 0.f, 0.f, 0.f), alo = ahi;
     double kick = 0.0, vx = 0.0, vy = 0.0, vz = 0.0;
+    const size_t ns = s.cl.on ? (size_t)s.cl.ncol * s.cl.maxcl * BOUNCE_CL : (size_t)s.n;
+    unsigned long long* acc = s.cl.on ? s.cl.acc : s.tl.acc;
+    const bool sums = !(ext && hout == 0.0);
     if (live) {
         if (s.cl.on) sl = s.cl.a2s[i];
-        if (!(ext && hout == 0.0)) {
-            const size_t ns = s.cl.on ? (size_t)s.cl.ncol * s.cl.maxcl * BOUNCE_CL : (size_t)s.n;
-            unsigned long long* acc = s.cl.on ? s.cl.acc : s.tl.acc;
-            gx = (float)((double)(long long)acc[sl] * CL_UNFIX);
-            gy = (float)((double)(long long)acc[ns + sl] * CL_UNFIX);
-            gz = (float)((double)(long long)acc[2 * ns + sl] * CL_UNFIX);
-            acc[sl] = 0ull;
-            acc[ns + sl] = 0ull;
-            acc[2 * ns + sl] = 0ull;
+        if (sums) {
+            gx = unfix32((long long)acc[sl]);
+            gy = unfix32((long long)acc[ns + sl]);
+            gz = unfix32((long long)acc[2 * ns + sl]);
         }
         Gx = ext ? 0.f : gx;
         Gy = ext ? 0.f : gy;
@@ -1011,9 +1011,9 @@ __global__ void __launch_bounds__(256, LITE_MIN_CTAS) k_step_lite(DevSys s, Para
     if (do_j2 && live) jump_lite(s, p, cur, i, step - 1, BOUNCE_STREAM_J2, ahi, alo, vx, vy, vz, nprop, nacc, near);
     if (live) {
         const double c = hk * kick;
-        vx -= c * (double)Gx;
-        vy -= c * (double)Gy;
-        vz -= c * (double)Gz;
+        vx -= c * widen(Gx);
+        vy -= c * widen(Gy);
+        vz -= c * widen(Gz);
         if (hr != 0.0) {
             const double cr = hr * kick;
             vx -= cr * s.grecip[i];
@@ -1022,16 +1022,38 @@ __global__ void __launch_bounds__(256, LITE_MIN_CTAS) k_step_lite(DevSys s, Para
         }
         if (ext && hout != 0.0) {
             const double co = hout * kick;
-            vx -= co * (double)gx;
-            vy -= co * (double)gy;
-            vz -= co * (double)gz;
+            vx -= co * widen(gx);
+            vy -= co * widen(gy);
+            vz -= co * widen(gz);
         }
     }
     if (do_j1 && live) jump_lite(s, p, cur, i, step, BOUNCE_STREAM_J1, ahi, alo, vx, vy, vz, nprop, nacc, near);
     if (live) {
         if (do_aoa) {
+            // everything that is read here is read before the first store: a
+            // store in between would hold the loads behind it back (they might
+            // alias for all the compiler knows), a trip to memory each
+            const double x0 = s.qx[cur][i], y0 = s.qy[cur][i], z0 = s.qz[cur][i], sd = s.osd[i];
+            double rx = 0.0, ry = 0.0, rz = 0.0, cx = 0.0, cy = 0.0, cz = 0.0, ox = 0.0, oy = 0.0, oz = 0.0;
+            float4 pr = ahi;
+            if (s.rows_flag) {
+                rx = s.refx[i];
+                ry = s.refy[i];
+                rz = s.refz[i];
+            }
+            if (s.cl.on) {
+                cx = s.cl.crefx[i];
+                cy = s.cl.crefy[i];
+                cz = s.cl.crefz[i];
+                if (p.periodic) {
+                    ox = s.cl.cofx[i];
+                    oy = s.cl.cofy[i];
+                    oz = s.cl.cofz[i];
+                }
+                pr = s.cl.pref[sl];
+            }
             const double h = 0.5 * p.dt;
-            double x = s.qx[cur][i] + h * vx, y = s.qy[cur][i] + h * vy, z = s.qz[cur][i] + h * vz;
+            double x = x0 + h * vx, y = y0 + h * vy, z = z0 + h * vz;
             // O: Box-Muller on Philox slot 0, stream 0
             const uint4 r = rng_atom(s, p, 0u, i, step, BOUNCE_STREAM_O);
             const float ra = sqrtf(-2.f * logf(u24_open0(r.x)));
@@ -1039,42 +1061,42 @@ __global__ void __launch_bounds__(256, LITE_MIN_CTAS) k_step_lite(DevSys s, Para
             sincospif(2.f * u24(r.y), &sn, &cs);
             const float n0 = ra * cs, n1 = ra * sn;
             const float n2 = sqrtf(-2.f * logf(u24_open0(r.z))) * cospif(2.f * u24(r.w));
-            const double sd = s.osd[i];
-            vx = p.c1 * vx + sd * (double)n0;
-            vy = p.c1 * vy + sd * (double)n1;
-            vz = p.c1 * vz + sd * (double)n2;
+            vx = p.c1 * vx + sd * widen(n0);
+            vy = p.c1 * vy + sd * widen(n1);
+            vz = p.c1 * vz + sd * widen(n2);
             x += h * vx;
             y += h * vy;
             z += h * vz;
-            s.qx[nxt][i] = x;
-            s.qy[nxt][i] = y;
-            s.qz[nxt][i] = z;
             double wx = x, wy = y, wz = z;
             if (p.periodic) {
                 wx = wrap_box(x, p.Ld[0], p.iLd[0]);
                 wy = wrap_box(y, p.Ld[1], p.iLd[1]);
                 wz = wrap_box(z, p.Ld[2], p.iLd[2]);
             }
-            const float hx = __double2float_rn(wx), hy = __double2float_rn(wy), hz = __double2float_rn(wz);
-            const float4 ph = make_float4(hx, hy, hz, ahi.w);
-            const float4 pl = make_float4(__double2float_rn(wx - (double)hx), __double2float_rn(wy - (double)hy),
-                                          __double2float_rn(wz - (double)hz), alo.w);
+            float4 ph, pl;
+            split_pos(wx, wy, wz, ahi.w, alo.w, ph, pl);
+            s.qx[nxt][i] = x;
+            s.qy[nxt][i] = y;
+            s.qz[nxt][i] = z;
             s.phi[nxt][i] = ph;
             s.plo[nxt][i] = pl;
-            const double ex = x - s.refx[i], ey = y - s.refy[i], ez = z - s.refz[i];
-            if (s.rows_flag && ((s.rows_move >> type_of(alo)) & 1) && ex * ex + ey * ey + ez * ez > p.skin_half2)
+            if (s.rows_flag && ((s.rows_move >> type_of(alo)) & 1) &&
+                moved_beyond(x - rx, y - ry, z - rz, p.skin_half2, p.skin_half2f))
                 atomicOr(s.rebuild, 1);
             if (s.cl.on) {
                 float4 ch = ph, cw = pl;
-                if (p.periodic) split_pos(x, y, z, s.cl.cofx[i], s.cl.cofy[i], s.cl.cofz[i], ph.w, pl.w, ch, cw);
+                if (p.periodic) split_pos(x - ox, y - oy, z - oz, ph.w, pl.w, ch, cw);
                 s.cl.sphi[nxt][sl] = ch;
                 s.cl.splo[nxt][sl] = cw;
-                const double cx = x - s.cl.crefx[i], cy = y - s.cl.crefy[i], cz = z - s.cl.crefz[i];
-                if (cx * cx + cy * cy + cz * cz > s.cl.cskin_half2) atomicOr(s.cl.rebuild, 1);
-                const float4 pr = s.cl.pref[sl];
+                if (moved_beyond(x - cx, y - cy, z - cz, s.cl.cskin_half2, s.cl.cskin_half2f)) atomicOr(s.cl.rebuild, 1);
                 const float px = ch.x - pr.x, py = ch.y - pr.y, pz = ch.z - pr.z;
                 if (px * px + py * py + pz * pz > s.cl.pdisp2) atomicOr(s.cl.prune, 1);
             }
+        }
+        if (sums) {  // cleared for the next evaluation
+            acc[sl] = 0ull;
+            acc[ns + sl] = 0ull;
+            acc[2 * ns + sl] = 0ull;
         }
         s.vx[i] = vx;
         s.vy[i] = vy;
@@ -1201,9 +1223,12 @@ void launch_step_kernel(const DevSys& s, const Params& p, int integrator, int va
     // from the cluster or tile kernel (or none at this boundary), and rare
     // proposals (s.lite, decided on the host from the jump bounds)
     if (s.lite && (s.cl.on || s.tl.on) && (pre || (ext && hout == 0.0))) {
-        const int lb = (s.n + 255) / 256;
-        if (integrator != 0) launch_chained(k_step_lite<1>, lb, 256, 0, st, s, p, variant, step_off, hr, ext, hout);
-        else launch_chained(k_step_lite<0>, lb, 256, 0, st, s, p, variant, step_off, hr, 0, 0.0);
+        const int lb = (s.n + LITE_T - 1) / LITE_T;
+        const bool few = lb <= 152 * LITE_FEW;
+        auto k = integrator != 0 ? (few ? k_step_lite<1, LITE_FEW> : k_step_lite<1, LITE_MANY>)
+                                 : (few ? k_step_lite<0, LITE_FEW> : k_step_lite<0, LITE_MANY>);
+        launch_chained(k, lb, LITE_T, 0, st, s, p, variant, step_off, hr, integrator != 0 ? ext : 0,
+                       integrator != 0 ? hout : 0.0);
         return;
     }
     if (integrator != 0)
