@@ -13,7 +13,7 @@
 // before (more warps in flight on the partners' gathers); short-row pair sums
 // stay in the step kernel.
 //
-// Work mapping (one CTA = 32 consecutive atoms, NW warps):
+// Work mapping (one CTA = grp <= 32 consecutive atoms, NW warps):
 //   * pair sums and jump proposals are warp-cooperative, lanes over
 //     neighbours / proposals, warps over the CTA's atoms;
 //   * every FP64 operation (B, A, O, ||v||, Poisson means, accumulation of
@@ -510,7 +510,7 @@ __device__ float3 atom_gradient(const DevSys& s, const Params& p, int cur, int i
 // boundaries, 0 elsewhere, where the pair sums are skipped).
 template <int BOUNCE>
 __global__ void __launch_bounds__(NW * 32, 3) k_step(DevSys s, Params p, int variant, int step_off, double hr,
-                                                     int ext, double hout, int pre) {
+                                                     int ext, double hout, int pre, int grp) {
     __shared__ float sG[BOUNCE_GROUP][3];
     __shared__ float sGp[BOUNCE_GROUP][3];
     __shared__ double sV[BOUNCE_GROUP][3];
@@ -525,8 +525,8 @@ __global__ void __launch_bounds__(NW * 32, 3) k_step(DevSys s, Params p, int var
     __shared__ float sNz[BOUNCE_GROUP][3], sU[2][BOUNCE_GROUP], sHw[BOUNCE_GROUP], sLw[BOUNCE_GROUP];
     chain_enter();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int base = blockIdx.x * BOUNCE_GROUP;
-    const int na = min(BOUNCE_GROUP, s.n - base);
+    const int base = blockIdx.x * grp;
+    const int na = min(grp, s.n - base);
     const long long step = *s.step_base + step_off;
     const int cur = (int)(step & 1), nxt = cur ^ 1;
     const bool do_j2 = BOUNCE && variant != 0;
@@ -1122,12 +1122,12 @@ __global__ void __launch_bounds__(LITE_T, CTAS) k_step_lite(const __grid_constan
 
 // One jump half-step on the current velocities (component entry point).
 __global__ void __launch_bounds__(NW * 32) k_jump_half(DevSys s, Params p, int cur, long long step, int stream_id,
-                                                      int* Mout, int* Aout) {
+                                                      int* Mout, int* Aout, int grp) {
     __shared__ JumpSmem js;
     __shared__ PropSmem ps;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int base = blockIdx.x * BOUNCE_GROUP;
-    const int na = min(BOUNCE_GROUP, s.n - base);
+    const int base = blockIdx.x * grp;
+    const int na = min(grp, s.n - base);
     if (threadIdx.x == 0) {
         js.cnt[0] = js.cnt[1] = js.cnt[2] = 0ull;
     }
@@ -1215,9 +1215,21 @@ int launch_step_pairs(const DevSys& s, const Params& p, int integrator, int step
     return pre;
 }
 
+// Atoms per CTA of the cooperative kernels: as few as leave all CTAs resident
+// at once (three an SM), at least two.  A CTA's eight warps share out its
+// atoms' pair sums and jump chains, so that fewer atoms are a shorter step:
+// 192 atoms with Coulomb on the jumps (dt 0.25 fs) 28 us a step with 32 of
+// them to a CTA, 22 with two; 1,800 atoms 47 with 32, 30 with four; 12,288
+// atoms 72 with 32, 87 with 16 in two waves.
+static int step_group(int n) {
+    int g = BOUNCE_GROUP;
+    while (g > 2 && (n + g / 2 - 1) / (g / 2) <= 152 * 3) g /= 2;
+    return g;
+}
+
 void launch_step_kernel(const DevSys& s, const Params& p, int integrator, int variant, int step_off, double hr,
                         double hout, int pre, cudaStream_t st) {
-    const int blocks = (s.n + BOUNCE_GROUP - 1) / BOUNCE_GROUP;
+    const int grp = step_group(s.n), blocks = (s.n + grp - 1) / grp;
     const int ext = integrator >= 3 ? 1 : 0;
     // the thread-per-atom kernel where its preconditions hold: pair sums
     // from the cluster or tile kernel (or none at this boundary), and rare
@@ -1232,8 +1244,8 @@ void launch_step_kernel(const DevSys& s, const Params& p, int integrator, int va
         return;
     }
     if (integrator != 0)
-        launch_chained(k_step<1>, blocks, NW * 32, 0, st, s, p, variant, step_off, hr, ext, hout, pre);
-    else launch_chained(k_step<0>, blocks, NW * 32, 0, st, s, p, variant, step_off, hr, 0, 0.0, pre);
+        launch_chained(k_step<1>, blocks, NW * 32, 0, st, s, p, variant, step_off, hr, ext, hout, pre, grp);
+    else launch_chained(k_step<0>, blocks, NW * 32, 0, st, s, p, variant, step_off, hr, 0, 0.0, pre, grp);
 }
 
 void launch_step(const DevSys& s, const Params& p, int integrator, int variant, int step_off, double hr,
@@ -1244,8 +1256,8 @@ void launch_step(const DevSys& s, const Params& p, int integrator, int variant, 
 
 void launch_jump_half(const DevSys& s, const Params& p, int cur, long long step, int stream_id, int* M, int* nacc,
                       cudaStream_t st) {
-    const int blocks = (s.n + BOUNCE_GROUP - 1) / BOUNCE_GROUP;
-    k_jump_half<<<blocks, NW * 32, 0, st>>>(s, p, cur, step, stream_id, M, nacc);
+    const int grp = step_group(s.n), blocks = (s.n + grp - 1) / grp;
+    k_jump_half<<<blocks, NW * 32, 0, st>>>(s, p, cur, step, stream_id, M, nacc, grp);
 }
 
 void launch_gradient(const DevSys& s, const Params& p, int part, int cur, double* out, cudaStream_t st) {

@@ -1,6 +1,9 @@
-"""The split FP32 positions that the step kernels leave (integer conversions)
-against those of a state set from outside (the conversion instructions): a
-comparison of bits.
+"""The step kernels where their launch shape and their conversions change:
+atom counts on both sides of each CTA size of the cooperative kernel (which
+then has 2, 4, 8, 16 or 32 atoms to a CTA) against the thread-per-atom kernel,
+whose result does not depend on it, and the split FP32 positions that the step
+kernels leave (integer conversions) against those of a state set from outside
+(the conversion instructions).  Both are comparisons of bits.
 """
 import numpy as np
 import pytest
@@ -10,6 +13,20 @@ pytestmark = pytest.mark.gpu
 from paper_2002_07109_gb300.water import water_box, water_droplet_molecules
 
 bounce = pytest.importorskip("paper_2002_07109_gb300.bounce")
+
+
+@pytest.mark.parametrize("n_mol", [1, 304, 305, 608, 609, 1216, 1217, 2432, 2433])
+def test_atoms_of_a_cooperative_cta(n_mol):
+    s = water_droplet_molecules(n_mol, seed=4)
+    out = []
+    for sk in (1, 2):
+        ctx = bounce.from_system(s, seed=5, r_on=3.0, r_off=4.0, jump_coulomb=False, max_neighbors=3 * n_mol, step_kernel=sk)
+        ctx.set_state(s.q, s.v, step=0)
+        ctx.run(3, bounce.BOUNCE)
+        e = ctx.energies()
+        out.append((*ctx.get_state(), e["proposals"], e["accepts"], e["near_ties"]))
+        ctx.close()
+    assert all(np.array_equal(a, b) for a, b in zip(*out))
 
 
 @pytest.mark.parametrize("sk", [1, 2])
