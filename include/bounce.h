@@ -338,7 +338,7 @@ int64_t bounce_run_launch_count(const bounce_ctx* ctx, int64_t n_steps, int32_t 
  * a DEVICE array of 2 doubles written on `stream`.  A type outside
  * [0, n_types) is not read from the tables: both totals are then NaN.
  * The call allocates nothing: its scratch is a static device array of
- * BOUNCE_NOALLOC_MAX_ATOMS atoms plus a status word (786,688 bytes) that
+ * BOUNCE_NOALLOC_MAX_ATOMS atoms plus status bytes (786,688 bytes) that
  * every GPU loading this library holds until exit.  n > BOUNCE_NOALLOC_MAX_ATOMS
  * returns BOUNCE_ERR_INVALID_ARG.  The first call on a device looks up the
  * scratch address on that device (make it before any stream capture).
