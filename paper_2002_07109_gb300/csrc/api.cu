@@ -676,7 +676,7 @@ int setup_clusters(bounce_ctx* c, const double* q, const HostBox& hb) {
     }
     int r;
     if (!c->cl_atoms_alloc) {
-        if ((r = dalloc(c, &nk.col_atoms, n)) || (r = dalloc(c, &nk.atom_col, n)) || (r = dalloc(c, &nk.a2s, n)) ||
+        if ((r = dalloc(c, &nk.col_atoms, n)) || (r = dalloc(c, &nk.a2s, n)) ||
             (r = dalloc(c, &nk.crefx, n)) || (r = dalloc(c, &nk.crefy, n)) || (r = dalloc(c, &nk.crefz, n)) ||
             (r = dalloc(c, &nk.cofx, n)) || (r = dalloc(c, &nk.cofy, n)) || (r = dalloc(c, &nk.cofz, n)) ||
             (r = dalloc(c, &nk.rebuild, 1)) || (r = dalloc(c, &nk.done_ctr, 4)) || (r = dalloc(c, &nk.prune, 1)) ||
@@ -801,12 +801,13 @@ void set_jump_partners(bounce_ctx* c, const std::vector<double>& sg, const std::
 // flag unless forced).  After BAOAB runs on clusters the step kernel did not
 // test the rows' displacement, so it is tested here first, at the current
 // positions (the test the oracle applies before every use of the rows).
+void rows_check(bounce_ctx* c, int step_off, cudaStream_t st) {
+    if (!c->rows_check_due) return;
+    if (step_off == 0) launch_flag_moved(c->ds, c->pp, (int)(c->cur_step & 1), st);
+    c->rows_check_due = false;
+}
 void rebuild(bounce_ctx* c, int step_off, bool force, cudaStream_t st, int mode = ROWS_ALL) {
-    if (c->rows_check_due) {
-        long long step = c->cur_step;
-        if (step_off == 0) launch_flag_moved(c->ds, c->pp, (int)(step & 1), st);
-        c->rows_check_due = false;
-    }
+    rows_check(c, step_off, st);
     launch_rebuild(c->ds, c->pp, step_off, force, c->bitmap_warps, c->bitmap_bytes, mode, st);
 }
 
@@ -995,8 +996,17 @@ double expected_proposals(bounce_ctx* c, double rho) {
 // the candidate rows, which only the jump step reads (BOUNCE integrators, or
 // every integrator without clusters, whose pair sums run over the rows).
 void rebuild_for(bounce_ctx* c, int integ, int off, cudaStream_t st) {
-    if (c->ds.cl.on) launch_cluster_rebuild(c->ds, c->pp, off, false, st);
-    if (!c->ds.cl.on || integ != BOUNCE_BAOAB) rebuild(c, off, false, st, run_rows_mode(c, integ));
+    if (c->ds.cl.on && integ != BOUNCE_BAOAB) {
+        const int mode = run_rows_mode(c, integ);
+        rows_check(c, off, st);
+        launch_bins(c->ds, c->pp, off, false, BIN_CELLS | BIN_COLUMNS, mode, st);
+        launch_cluster_rebuild(c->ds, c->pp, off, false, st, true);
+        launch_rebuild(c->ds, c->pp, off, false, c->bitmap_warps, c->bitmap_bytes, mode, st, true);
+    } else if (c->ds.cl.on) {
+        launch_cluster_rebuild(c->ds, c->pp, off, false, st);
+    } else {
+        rebuild(c, off, false, st, run_rows_mode(c, integ));
+    }
 }
 
 // Before a run: rows a previous run left partial are completed when this
@@ -1632,13 +1642,13 @@ int bounce_autotune(bounce_ctx* c, int32_t integ, void* stream, bounce_tuning* o
 
 int64_t bounce_run_launch_count(const bounce_ctx* c, int64_t n, int32_t integ) {
     if (!c || n <= 0) return 0;
-    // gated row-rebuild kernels (cells count + scan, scatter, rows + flag clear;
-    // one kernel for a batch of replicas) + the fused step kernel, and the
+    // gated rebuild kernels + the fused step kernel, and the
     // pair-sum kernel wherever the boundary has pair sums over the long rows
     const bool clu = c->ds.cl.on != 0;
-    // gated rebuilds: the clusters (4, and the list prune), the rows (3, or 1
-    // for a batch) unless BAOAB runs on clusters; then the step kernel
-    const int64_t per_boundary = (clu ? 5 : 0) + ((clu && integ == BOUNCE_BAOAB) ? 0 : (c->ds.rep_of ? 1 : 3)) + 1;
+    // gated rebuilds: the bins (none in a batch), the clusters (sort, lists),
+    // the rows unless BAOAB runs on clusters; then the step kernel
+    const int64_t per_boundary =
+        (c->ds.rep_of ? 0 : 1) + (clu ? 2 : 0) + ((clu && integ == BOUNCE_BAOAB) ? 0 : 1) + 1;
     const bool ext = integ >= BOUNCE_BOUNCE_RESPA_EXT;
     const bool short_f0 = !clu && integ != BOUNCE_BAOAB && c->pp.rshort2 < INFINITY;
     const int64_t pme_launches = c->has_pme ? pme_launch_count(c->pme) : 0;

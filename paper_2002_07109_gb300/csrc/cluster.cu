@@ -70,91 +70,13 @@ __device__ bool cl_last_cta(unsigned int* ctr) {
     return last;
 }
 
-// Exclusive block-wide scan of x over all threads of the CTA (blockDim a
-// multiple of 32, at most 1024); returns the prefix, *total the sum.
-__device__ int block_scan(int x, int* total) {
-    __shared__ int wsum[32];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    int v = x;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v += y;
-    }
-    if (lane == 31) wsum[w] = v;
-    __syncthreads();
-    if (w == 0) {
-        int t = lane < nw ? wsum[lane] : 0;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, t, o);
-            if (lane >= o) t += y;
-        }
-        wsum[lane] = t;
-    }
-    __syncthreads();
-    const int excl = (w > 0 ? wsum[w - 1] : 0) + v - x;
-    *total = wsum[nw - 1];
-    __syncthreads();
-    return excl;
-}
-
-__device__ __forceinline__ int column_of(const DevClu& c, const Params& p, float4 hi) {
-    int cx, cy;
-    if (p.periodic) {
-        cx = min(max((int)(hi.x * c.ihx), 0), c.ncx - 1);
-        cy = min(max((int)(hi.y * c.ihy), 0), c.ncy - 1);
-    } else {
-        cx = min(max((int)floorf((hi.x - c.ox) * c.ihx), 0), c.ncx - 1);
-        cy = min(max((int)floorf((hi.y - c.oy) * c.ihy), 0), c.ncy - 1);
-    }
-    return cy * c.ncx + cx;
-}
-
-// 1. columns and their counts; the last CTA scans them.
-__global__ void k_cl_count(DevSys s, Params p, int step_off, int force) {
-    if (!cl_pending(s, force)) return;
-    const DevClu& c = s.cl;
-    const int cur = (int)((*s.step_base + step_off) & 1);
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < s.n; i += gridDim.x * blockDim.x) {
-        const int col = column_of(c, p, s.phi[cur][i]);
-        c.atom_col[i] = col;
-        atomicAdd(&c.col_count[col], 1);
-    }
-    if (!cl_last_cta(&c.done_ctr[0])) return;
-    int carry = 0;
-    for (int b = 0; b < c.ncol; b += blockDim.x) {
-        const int col = b + threadIdx.x;
-        const int v = col < c.ncol ? __ldcg(&c.col_count[col]) : 0;
-        int tot;
-        const int ex = block_scan(v, &tot);
-        if (col < c.ncol) {
-            c.col_start[col] = carry + ex;
-            c.col_fill[col] = carry + ex;
-            c.col_count[col] = 0;
-        }
-        carry += tot;
-    }
-    if (threadIdx.x == 0) c.col_start[c.ncol] = carry;
-}
-
-// 2. atom indices in column order (arbitrary order inside a column).
-__global__ void k_cl_scatter(DevSys s, Params p, int step_off, int force) {
-    if (!cl_pending(s, force)) return;
-    const DevClu& c = s.cl;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < s.n; i += gridDim.x * blockDim.x) {
-        const int pos = atomicAdd(&c.col_fill[c.atom_col[i]], 1);
-        c.col_atoms[pos] = i;
-    }
-}
-
 // Order-preserving map of a float onto an unsigned key.
 __device__ __forceinline__ uint32_t float_key(float z) {
     const uint32_t b = __float_as_uint(z);
     return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
 }
 
-// 3. one CTA per column: sort by (z, index), clusters, slots, boxes.
+// 2. one CTA per column (binned by k_bins): sort by (z, index), clusters, slots, boxes.
 __global__ void __launch_bounds__(SORT_NT) k_cl_sort(DevSys s, Params p, int step_off, int force) {
     if (!cl_pending(s, force)) return;
     __shared__ unsigned long long key[BOUNCE_CL_MAXCOL];
@@ -269,7 +191,7 @@ __device__ __forceinline__ void shift_split(float& h, float& l, float sh, float 
     l = (l - sl) + err;
 }
 
-// 4. neighbour lists (CTA per cluster I): every atom j of a cluster
+// 3a. neighbour lists (CTA per cluster I): every atom j of a cluster
 // J >= I of the columns in reach whose distance to I's bounding box (minimum
 // image per axis) is below the search radius, in a fixed order, as its slot
 // with the periodic image of the pair (or the per-pair code when the pair's
@@ -292,8 +214,7 @@ constexpr int NB_PASS = 4;                     // atoms (entries) in flight per 
 constexpr int NB_QUEUE = NB_PASS * NB_NT / CL;  // clusters of an atom-level step
 constexpr int NB_RING = 256;                   // queued clusters: < NB_QUEUE left over + 128 new
 
-__global__ void __launch_bounds__(NB_NT, 8) k_cl_search(DevSys s, Params p, int step_off, int force) {
-    if (!cl_pending(s, force)) return;
+__device__ __forceinline__ void cl_search(const DevSys& s, const Params& p, int step_off) {
     __shared__ int run_start[NB_NT], run_off[NB_NT];  // non-empty columns: first candidate, first cluster less it
     __shared__ int wsum[NB_W];
     __shared__ int ring[NB_RING];
@@ -485,11 +406,6 @@ __global__ void __launch_bounds__(NB_NT, 8) k_cl_search(DevSys s, Params p, int 
         overflow = overflow || m0 > c.capj[0] || (c.nlists > 1 && m1 > c.capj[1]);
     }
     if (overflow && tid == 0) atomicOr(s.err, BERR_LIST_OVERFLOW);
-    if (!cl_last_cta(&c.done_ctr[1])) return;
-    if (threadIdx.x == 0) {
-        *c.rebuild = 0;
-        *c.prune = 1;  // new lists: prune them before the next pair sums
-    }
 }
 
 // Whether list entry `ent` (high part hj of the j atom's slot copy) lies
@@ -522,7 +438,7 @@ __device__ __forceinline__ bool prune_keep(const DevSys& s, const Params& p, int
     return best < R2;
 }
 
-// 5. pruned lists (warp per cluster I), gated by the prune flag: the
+// 3b. pruned lists (warp per cluster I): the
 // entries of each list whose atom j lies within the prune radius of at least
 // one atom of I at the current positions (same images as the pair kernel;
 // FP32 with a margin, so that no pair the exact test would keep is dropped),
@@ -532,16 +448,28 @@ __device__ __forceinline__ bool prune_keep(const DevSys& s, const Params& p, int
 // Bounded by the chain of one list (entries, their positions, the vote): four
 // passes of 32 entries are in flight per warp (two: 30 us for 12,288 atoms, 73 us
 // for 98,304; four: 26 and 67).  A CTA per cluster takes 24 and 98 us.
-__global__ void __launch_bounds__(NB_NT, 8) k_cl_prune(DevSys s, Params p, int step_off, int force) {
+//
+// 3. The two in one launch: a CTA prunes the clusters whose lists it has just
+// made (new lists), or those it would make (prune flag alone).  Each kernel of
+// the gated sequence costs a step ~1.1 us when nothing is due.  (Apart, two
+// launches are no faster where both are due: 1447 against 1421 us for the
+// forces of two frames of 27,783 atoms.)
+__global__ void __launch_bounds__(NB_NT, 8) k_cl_lists(const __grid_constant__ DevSys s, const __grid_constant__ Params p,
+                                                       int step_off, int force) {
     chain_enter();
-    if (!(force || *s.cl.prune)) return;
     const DevClu& c = s.cl;
+    const bool search = force || *c.rebuild;
+    if (!(search || *c.prune)) return;
+    if (search) {
+        cl_search(s, p, step_off);
+        __syncthreads();  // the CTA's lists are written
+    }
     const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
     __shared__ float4 s_hi[NB_W][CL], s_lo[NB_W][CL];
     const int ncl = c.ncol * c.maxcl;
     const int cur = (int)((*s.step_base + step_off) & 1);
     const uint32_t below = (1u << lane) - 1u;
-    for (int t = blockIdx.x * NB_W + wl; t < ncl; t += gridDim.x * NB_W) {
+    for (int t = blockIdx.x + wl * gridDim.x; t < ncl; t += gridDim.x * NB_W) {
         const int kt = t / c.ncol, I = (t - kt * c.ncol) * c.maxcl + kt;  // the columns' unused slots come last
         int n[2];
         n[0] = c.lcnt[0][I];
@@ -596,14 +524,17 @@ __global__ void __launch_bounds__(NB_NT, 8) k_cl_prune(DevSys s, Params p, int s
             }
         }
     }
-    if (!cl_last_cta(&c.done_ctr[2])) return;
+    if (!cl_last_cta(&c.done_ctr[1])) return;
     if (threadIdx.x < 2) {
         const int L = threadIdx.x;
         const int n = atomicExch(&c.pnitems[2 + L], 0);
         c.pnitems[L] = min(n, c.capitems);
         if (n > c.capitems) atomicOr(s.err, BERR_LIST_OVERFLOW);
     }
-    if (threadIdx.x == 0) *c.prune = 0;
+    if (threadIdx.x == 0) {
+        *c.prune = 0;
+        if (search) *c.rebuild = 0;
+    }
 }
 
 // The pairs of one list entry (atom slot sj, split position hj/lj in the
@@ -793,15 +724,12 @@ __global__ void k_cl_collect(DevSys s, double* out) {
 
 }  // namespace
 
-void launch_cluster_rebuild(const DevSys& s, const Params& p, int step_off, bool force, cudaStream_t st) {
+void launch_cluster_rebuild(const DevSys& s, const Params& p, int step_off, bool force, cudaStream_t st, bool binned) {
     const int f = force ? 1 : 0;
-    const int tb = 1024, gb = (s.n + tb - 1) / tb;
-    launch_chained(k_cl_count, gb, tb, 0, st, s, p, step_off, f);
-    launch_chained(k_cl_scatter, gb, tb, 0, st, s, p, step_off, f);
+    if (!binned) launch_bins(s, p, step_off, force, BIN_COLUMNS, ROWS_ALL, st);
     launch_chained(k_cl_sort, std::min(s.cl.ncol, 152 * 8), SORT_NT, 0, st, s, p, step_off, f);
     const int ncl = s.cl.ncol * s.cl.maxcl;
-    launch_chained(k_cl_search, std::min(ncl, 152 * 8), NB_NT, 0, st, s, p, step_off, f);
-    launch_chained(k_cl_prune, std::min((ncl + NB_W - 1) / NB_W, 152 * 8), NB_NT, 0, st, s, p, step_off, f);
+    launch_chained(k_cl_lists, std::min(ncl, 152 * 8), NB_NT, 0, st, s, p, step_off, f);
 }
 
 // CTAs of a pair kernel that fit on the GPU at once (the warps fetch their

@@ -58,7 +58,6 @@ struct DevClu {
     int* col_fill;           // [ncol]
     int* col_atoms;          // [n] atoms in column order
     int* col_ncl;            // [ncol] clusters of each column
-    int* atom_col;           // [n] column of each atom at the build
     int* cl_atom;            // [ncl * CL] atom of each slot (-1: padding)
     int* a2s;                // [n] slot of each atom
     float4* sphi[2];         // slot-ordered copies of phi / plo (same buffers as the positions)
@@ -721,8 +720,13 @@ inline cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 bloc
 constexpr int ROWS_ALL = 0, ROWS_ACTIVE = 1, ROWS_IDLE = 2, ROWS_READER = 3, ROWS_FILTER = 8;
 
 // Launchers implemented in the .cu files.
+// The atoms binned into the cells of the rows, the columns of the clusters or
+// both (each gated by its flag), the first part of launch_rebuild and
+// launch_cluster_rebuild, which leave it out where it is done (binned).
+constexpr int BIN_CELLS = 1, BIN_COLUMNS = 2;
+void launch_bins(const DevSys& s, const Params& p, int step_off, bool force, int which, int mode, cudaStream_t st);
 void launch_rebuild(const DevSys& s, const Params& p, int step_off, bool force, int window_words, size_t bitmap_bytes,
-                    int mode, cudaStream_t st);
+                    int mode, cudaStream_t st, bool binned = false);
 void launch_step(const DevSys& s, const Params& p, int integrator, int variant, int step_off, double hr,
                  double hout, cudaStream_t st);
 // launch_step in two parts (for per-kernel timing): the pair sums, then the step kernel.
@@ -751,7 +755,8 @@ void launch_flag_moved(const DevSys& s, const Params& p, int cur, cudaStream_t s
 // the pair sums of `part` (3: F_0 share, 5: full pairs) over list `list`
 // into the fixed-point accumulators, and their read-out (added to out[3n],
 // accumulators cleared).
-void launch_cluster_rebuild(const DevSys& s, const Params& p, int step_off, bool force, cudaStream_t st);
+void launch_cluster_rebuild(const DevSys& s, const Params& p, int step_off, bool force, cudaStream_t st,
+                            bool binned = false);
 // sizes the pair kernel's resident grid once (outside any graph capture)
 void prepare_cluster_pairs();
 void launch_cluster_pairs(const DevSys& s, const Params& p, int step_off, int part, int list, cudaStream_t st);

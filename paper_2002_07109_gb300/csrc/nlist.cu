@@ -16,10 +16,9 @@
 // spatial order).
 // Every kernel returns at once unless a rebuild is pending (the step kernel
 // raises the flag when an atom has moved more than skin/2 since the last
-// build), so the sequence can sit in a captured CUDA graph.  Three launches:
-// cell counts (the CTA finishing last scans them), scatter into cell order
-// (indices, positions and molecule ids), rows (the CTA finishing last clears
-// the flag).
+// build), so the sequence can sit in a captured CUDA graph.  Two launches:
+// k_bins (counts, scan, scatter into cell order; it bins the clusters' columns
+// too), rows (the CTA finishing last clears the flag).
 #include <algorithm>
 
 #include "common.cuh"
@@ -27,6 +26,7 @@
 namespace {
 
 constexpr int ROWS_T = 128, ROWS_CTAS = 7;  // threads of a row CTA, CTAs of an SM (72 registers)
+constexpr int BIN_CTAS = 8, BIN_NT = 1024, BIN_PASS = 4;  // k_bins: CTAs, threads of each, atoms in flight per thread
 constexpr int RANGE_MAX = 128;  // cell-row runs per atom (<= 2 (2*3+1)^2 = 98)
 
 // Entry of a gated rebuild kernel: after its predecessor in the chain, is a
@@ -63,76 +63,149 @@ __device__ bool last_cta(unsigned int* ctr) {
     return last;
 }
 
-// Exclusive scan of the cell counts by one CTA; resets the counts to zero
-// for the next rebuild.
-__device__ void cells_scan(const DevSys& s) {
+// Exclusive scan of nc counts by one CTA into start (nc + 1 values) and fill;
+// resets the counts to zero for the next rebuild.  Four counts to a thread, in
+// one word of 16 bytes: the 10,000 cells of a box of 27,783 atoms are three
+// trips to memory, not ten.
+__device__ void bins_scan(int* count, int* start, int* fill, int nc) {
     __shared__ int warp_tot[32];
-    __shared__ int carry;
-    int nc = s.ncx * s.ncy * s.ncz;
-    if (threadIdx.x == 0) carry = 0;
-    __syncthreads();
-    for (int base = 0; base < nc; base += blockDim.x) {
-        int c = base + threadIdx.x;
-        int v = c < nc ? __ldcg(&s.cell_count[c]) : 0;  // written by other CTAs' atomics
-        int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-        int x = v;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    int carry = 0;
+    for (int base = 0; base < nc; base += BIN_NT * 4) {
+        const int c0 = base + threadIdx.x * 4;
+        const bool whole = c0 + 4 <= nc;
+        int4 v = make_int4(0, 0, 0, 0);  // (read past L1: written by other CTAs' atomics)
+        if (whole) {
+            v = __ldcg((const int4*)(count + c0));
+        } else if (c0 < nc) {
+            v.x = __ldcg(count + c0);
+            if (c0 + 1 < nc) v.y = __ldcg(count + c0 + 1);
+            if (c0 + 2 < nc) v.z = __ldcg(count + c0 + 2);
+        }
+        const int sum = v.x + v.y + v.z + v.w;
+        int x = sum;
         for (int o = 1; o < 32; o <<= 1) {
             int y = __shfl_up_sync(0xffffffffu, x, o);
             if (lane >= o) x += y;
         }
         if (lane == 31) warp_tot[w] = x;
         __syncthreads();
-        if (w == 0) {
-            int t = lane < (int)(blockDim.x >> 5) ? warp_tot[lane] : 0;
-            for (int o = 1; o < 32; o <<= 1) {
-                int y = __shfl_up_sync(0xffffffffu, t, o);
-                if (lane >= o) t += y;
-            }
-            warp_tot[lane] = t;
+        int t = warp_tot[lane];  // (BIN_NT / 32 = 32 warps)
+        for (int o = 1; o < 32; o <<= 1) {
+            int y = __shfl_up_sync(0xffffffffu, t, o);
+            if (lane >= o) t += y;
         }
-        __syncthreads();
-        int excl = carry + (w > 0 ? warp_tot[w - 1] : 0) + x - v;
-        if (c < nc) {
-            s.cell_start[c] = excl;
-            s.cell_fill[c] = excl;
-            s.cell_count[c] = 0;
+        const int before = __shfl_sync(0xffffffffu, t, max(w - 1, 0));
+        int4 e;
+        e.x = carry + x - sum + (w ? before : 0);
+        e.y = e.x + v.x;
+        e.z = e.y + v.y;
+        e.w = e.z + v.z;
+        carry += __shfl_sync(0xffffffffu, t, 31);
+        if (whole) {
+            *(int4*)(start + c0) = e;
+            *(int4*)(fill + c0) = e;
+            *(int4*)(count + c0) = make_int4(0, 0, 0, 0);
+        } else if (c0 < nc) {
+            const int f[3] = {e.x, e.y, e.z};
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+                if (c0 + k < nc) {
+                    start[c0 + k] = f[k];
+                    fill[c0 + k] = f[k];
+                    count[c0 + k] = 0;
+                }
         }
-        __syncthreads();
-        if (threadIdx.x == blockDim.x - 1) carry = excl + v;
-        __syncthreads();
+        __syncthreads();  // warp_tot is read
     }
-    if (threadIdx.x == 0) s.cell_start[nc] = carry;
+    if (threadIdx.x == 0) start[nc] = carry;
 }
 
-// Cell counts; the CTA that finishes last scans them.
 // Atom i goes into the cells (ROWS_FILTER: only the types some jump row can hold).
 __device__ __forceinline__ bool in_cells(const DevSys& s, const Params& p, int mode, int i) {
     return !(mode & ROWS_FILTER) || ((p.jcells >> s.type[i]) & 1);
 }
 
-__global__ void k_cells_count(DevSys s, Params p, int step_off, int force, int mode) {
-    if (!pending(s, force)) return;
-    int cur = (int)((*s.step_base + step_off) & 1);
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < s.n; i += gridDim.x * blockDim.x) {
-        if (!in_cells(s, p, mode, i)) continue;
-        int cx, cy, cz;
-        cell_of(s, p, s.phi[cur][i], cx, cy, cz);
-        atomicAdd(&s.cell_count[(cz * s.ncy + cy) * s.ncx + cx], 1);
+__device__ __forceinline__ int column_of(const DevClu& c, const Params& p, float4 hi) {
+    int cx, cy;
+    if (p.periodic) {
+        cx = min(max((int)(hi.x * c.ihx), 0), c.ncx - 1);
+        cy = min(max((int)(hi.y * c.ihy), 0), c.ncy - 1);
+    } else {
+        cx = min(max((int)floorf((hi.x - c.ox) * c.ihx), 0), c.ncx - 1);
+        cy = min(max((int)floorf((hi.y - c.oy) * c.ihy), 0), c.ncy - 1);
     }
-    if (last_cta(&s.done_ctr[0])) cells_scan(s);
+    return cy * c.ncx + cx;
 }
 
-__global__ void k_cells_scatter(DevSys s, Params p, int step_off, int force, int mode) {
-    if (!pending(s, force)) return;
-    int cur = (int)((*s.step_base + step_off) & 1);
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < s.n; i += gridDim.x * blockDim.x) {
-        if (!in_cells(s, p, mode, i)) continue;
+// All threads of a cluster of CTAs; what they wrote before is visible after it.
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Counting sort of the atoms into the row builder's cells (BIN_CELLS) and the
+// clusters' columns (BIN_COLUMNS, arbitrary order inside a column), gated by
+// their own flags: counts, their scan and the scatter in one launch, a
+// cluster of eight CTAs for each of the two, whose barriers part the phases.
+// The two counts, the two scatters and their launches apart cost a step four
+// gates of ~1.1 us when nothing is due.
+__global__ void __launch_bounds__(BIN_NT) k_bins(const __grid_constant__ DevSys s, const __grid_constant__ Params p,
+                                                 int step_off, int force, int which, int mode) {
+    chain_enter();
+    const bool columns = which == BIN_COLUMNS || blockIdx.x >= BIN_CTAS;
+    if (!(force || *(columns ? s.cl.rebuild : s.rebuild))) return;  // the same for the whole cluster
+    const int rank = blockIdx.x % BIN_CTAS, cur = (int)((*s.step_base + step_off) & 1);
+    const DevClu& c = s.cl;
+    int* count = columns ? c.col_count : s.cell_count;
+    int* fill = columns ? c.col_fill : s.cell_fill;
+    auto bin_of = [&](int i, float4 hi) {
+        if (columns) return column_of(c, p, hi);
         int cx, cy, cz;
-        const float4 hi = s.phi[cur][i];
         cell_of(s, p, hi, cx, cy, cz);
-        int pos = atomicAdd(&s.cell_fill[(cz * s.ncy + cy) * s.ncx + cx], 1);
-        s.cell_phi[pos] = make_float4(hi.x, hi.y, hi.z, __int_as_float(i));
-        s.cell_mt[pos] = make_int2(s.mol[i], s.type[i]);
+        return (cz * s.ncy + cy) * s.ncx + cx;
+    };
+    constexpr int STEP = BIN_CTAS * BIN_NT;
+    for (int i0 = rank * BIN_NT + threadIdx.x; i0 < s.n; i0 += BIN_PASS * STEP) {
+        int b[BIN_PASS];
+#pragma unroll
+        for (int u = 0; u < BIN_PASS; ++u) {
+            const int i = i0 + u * STEP;
+            b[u] = i < s.n && (columns || in_cells(s, p, mode, i)) ? bin_of(i, s.phi[cur][i]) : -1;
+        }
+#pragma unroll
+        for (int u = 0; u < BIN_PASS; ++u)
+            if (b[u] >= 0) atomicAdd(&count[b[u]], 1);
+    }
+    cluster_sync();
+    if (rank == 0)
+        bins_scan(count, columns ? c.col_start : s.cell_start, fill, columns ? c.ncol : s.ncx * s.ncy * s.ncz);
+    cluster_sync();
+    for (int i0 = rank * BIN_NT + threadIdx.x; i0 < s.n; i0 += BIN_PASS * STEP) {
+        int b[BIN_PASS];
+        float4 hi[BIN_PASS];
+#pragma unroll
+        for (int u = 0; u < BIN_PASS; ++u) {
+            const int i = i0 + u * STEP;
+            b[u] = -1;
+            if (i < s.n && (columns || in_cells(s, p, mode, i))) {
+                hi[u] = s.phi[cur][i];
+                b[u] = bin_of(i, hi[u]);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < BIN_PASS; ++u)
+            if (b[u] >= 0) b[u] = atomicAdd(&fill[b[u]], 1);
+#pragma unroll
+        for (int u = 0; u < BIN_PASS; ++u) {
+            const int i = i0 + u * STEP;
+            if (b[u] < 0) continue;
+            if (columns) {
+                c.col_atoms[b[u]] = i;
+            } else {
+                s.cell_phi[b[u]] = make_float4(hi[u].x, hi[u].y, hi[u].z, __int_as_float(i));
+                s.cell_mt[b[u]] = make_int2(s.mol[i], s.type[i]);
+            }
+        }
     }
 }
 
@@ -683,8 +756,24 @@ void launch_flag_moved(const DevSys& s, const Params& p, int cur, cudaStream_t s
     k_flag_moved<<<(s.n + 255) / 256, 256, 0, st>>>(s, p, cur);
 }
 
+void launch_bins(const DevSys& s, const Params& p, int step_off, bool force, int which, int mode, cudaStream_t st) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = which == (BIN_CELLS | BIN_COLUMNS) ? 2 * BIN_CTAS : BIN_CTAS;
+    cfg.blockDim = BIN_NT;
+    cfg.stream = st;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = BIN_CTAS;
+    at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+    cudaLaunchKernelEx(&cfg, k_bins, s, p, step_off, force ? 1 : 0, which, mode);
+}
+
 void launch_rebuild(const DevSys& s, const Params& p, int step_off, bool force, int window_words, size_t bitmap_bytes,
-                    int mode, cudaStream_t st) {
+                    int mode, cudaStream_t st, bool binned) {
     const int f = force ? 1 : 0;
     if (s.rep_of) {
         const int wpb = 8;
@@ -693,10 +782,7 @@ void launch_rebuild(const DevSys& s, const Params& p, int step_off, bool force, 
         launch_chained(k_rows_batch, std::min((s.n + wpb - 1) / wpb, 152 * 8), wpb * 32, 0, st, s, p, step_off, f, mode);
         return;
     }
-    const int tb = 1024;
-    const int gb = (s.n + tb - 1) / tb;
-    launch_chained(k_cells_count, gb, tb, 0, st, s, p, step_off, f, mode);
-    launch_chained(k_cells_scatter, gb, tb, 0, st, s, p, step_off, f, mode);
+    if (!binned) launch_bins(s, p, step_off, force, BIN_CELLS, mode, st);
     // Warp per atom, a grid-stride loop over one wave of CTAs where the launch may find nothing to do; a forced
     // build takes up to four waves, so that an SM which is done early gets another CTA (27,783 atoms: 196 -> 175 us).
     // CTAs of four warps, not eight: 418 -> 392 us there, 87.4 -> 84.0 us on 12,288 atoms.
