@@ -957,7 +957,12 @@ __global__ void __launch_bounds__(LITE_T, CTAS) k_step_lite(const __grid_constan
                                                                    const __grid_constant__ Params p, int variant,
                                                                    int step_off, double hr, int ext, double hout) {
     __shared__ unsigned long long cnt[4];
-    chain_enter();
+    // Where the kernel before is the pair kernel, only its sums are waited for:
+    // it began after every other kernel of the chain had ended (chain_enter),
+    // so the atoms' state and the bonded terms are read and evaluated while
+    // its last warps still work.
+    const bool sums = !(ext && hout == 0.0);
+    if (!sums) chain_enter();
     if (threadIdx.x < 4) cnt[threadIdx.x] = 0ull;
     const int lane = threadIdx.x & 31;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -977,35 +982,34 @@ __global__ void __launch_bounds__(LITE_T, CTAS) k_step_lite(const __grid_constan
     double kick = 0.0, vx = 0.0, vy = 0.0, vz = 0.0;
     const size_t ns = s.cl.on ? (size_t)s.cl.ncol * s.cl.maxcl * BOUNCE_CL : (size_t)s.n;
     unsigned long long* acc = s.cl.on ? s.cl.acc : s.tl.acc;
-    const bool sums = !(ext && hout == 0.0);
+    float bx = 0.f, by = 0.f, bz = 0.f;
     if (live) {
         if (s.cl.on) sl = s.cl.a2s[i];
-        if (sums) {
-            gx = unfix32((long long)acc[sl]);
-            gy = unfix32((long long)acc[ns + sl]);
-            gz = unfix32((long long)acc[2 * ns + sl]);
-        }
-        Gx = ext ? 0.f : gx;
-        Gy = ext ? 0.f : gy;
-        Gz = ext ? 0.f : gz;
-        // bonded terms of the atom, in list order
-        float bx = 0.f, by = 0.f, bz = 0.f;
-        for (int t = s.bt_off[i]; t < s.bt_off[i + 1]; ++t) {
-            const float3 g = bonded_grad(p, s, cur, i, s.bt_idx[t], s.bt_par[t]);
-            bx += g.x;
-            by += g.y;
-            bz += g.z;
-        }
-        Gx += bx;
-        Gy += by;
-        Gz += bz;
         ahi = s.phi[cur][i];
         alo = s.plo[cur][i];
         kick = s.kick[i];
         vx = s.vx[i];
         vy = s.vy[i];
         vz = s.vz[i];
+        // bonded terms of the atom, in list order
+        for (int t = s.bt_off[i]; t < s.bt_off[i + 1]; ++t) {
+            const float3 g = bonded_grad(p, s, cur, i, s.bt_idx[t], s.bt_par[t]);
+            bx += g.x;
+            by += g.y;
+            bz += g.z;
+        }
     }
+    if (sums) {
+        chain_enter();
+        if (live) {
+            gx = unfix32((long long)acc[sl]);
+            gy = unfix32((long long)acc[ns + sl]);
+            gz = unfix32((long long)acc[2 * ns + sl]);
+        }
+    }
+    Gx = (ext ? 0.f : gx) + bx;
+    Gy = (ext ? 0.f : gy) + by;
+    Gz = (ext ? 0.f : gz) + bz;
     // the jump half-steps, one thread per atom: most atoms settle M = 0 from
     // their first draw (jump_thread), so no compaction or barrier pays off
     if (do_j2 && live) jump_lite(s, p, cur, i, step - 1, BOUNCE_STREAM_J2, ahi, alo, vx, vy, vz, nprop, nacc, near);
