@@ -1525,7 +1525,7 @@ int bounce_profile_breakdown(bounce_ctx* c, int64_t n_steps, int32_t integ, void
         ok = ok && mark(2);
         if (pme) launch_pme(c->ds, c->pp, c->pme, off, st);
         ok = ok && mark(4);
-        const int pre = launch_step_pairs(v, c->pp, integ, off, hout, st);
+        const int pre = launch_step_pairs(v, c->pp, integ, off, hr, hout, st);
         ok = ok && mark(0);
         launch_step_kernel(v, c->pp, integ, variant, off, hr, hout, pre, st);
         ok = ok && mark(1);

@@ -590,8 +590,9 @@ template <int PART, bool EW, bool CJ>
 __global__ void __launch_bounds__(PAIRS_NT, PAIRS_CTAS) k_cl_pairs(const __grid_constant__ DevSys s,
                                                                    const __grid_constant__ Params p,
                                                                    const __grid_constant__ PairConsts k, int step_off,
-                                                                   int L) {
-    chain_enter();
+                                                                   int L, int early) {
+    if (early) chain_next();
+    else chain_enter();
     __shared__ IGroup s_g[PAIRS_NT / 32];
     const DevClu& c = s.cl;
     const int lane = threadIdx.x & 31;
@@ -701,6 +702,7 @@ __global__ void __launch_bounds__(PAIRS_NT, PAIRS_CTAS) k_cl_pairs(const __grid_
             w = wn;
         }
     }
+    if (early) chain_wait();
     npair = warp_sum_i(npair);
     if (lane == 0 && npair) atomicAdd(&s.cnt[PART == 3 ? CNT_SHORT_PAIRS : CNT_FULL_PAIRS], (unsigned long long)npair);
     // every warp has seen the counter past the last item: the last CTA resets it
@@ -762,19 +764,20 @@ void prepare_cluster_pairs() {
 }
 
 template <int PART, bool CJ>
-static void launch_cl_pairs(const DevSys& s, const Params& p, int step_off, int list, cudaStream_t st) {
+static void launch_cl_pairs(const DevSys& s, const Params& p, int step_off, int list, bool early, cudaStream_t st) {
     const PairConsts k = make_pair_consts(p);
+    const int e = early ? 1 : 0;
     if (p.ebeta > 0.f)
-        launch_chained(k_cl_pairs<PART, true, CJ>, cl_pairs_grid<PART, true, CJ>(), PAIRS_NT, 0, st, s, p, k, step_off, list);
+        launch_chained(k_cl_pairs<PART, true, CJ>, cl_pairs_grid<PART, true, CJ>(), PAIRS_NT, 0, st, s, p, k, step_off, list, e);
     else
         launch_chained(k_cl_pairs<PART, false, CJ>, cl_pairs_grid<PART, false, CJ>(), PAIRS_NT, 0, st, s, p, k, step_off,
-                       list);
+                       list, e);
 }
 
-void launch_cluster_pairs(const DevSys& s, const Params& p, int step_off, int part, int list, cudaStream_t st) {
-    if (part != 3) launch_cl_pairs<5, true>(s, p, step_off, list, st);
-    else if (p.coul_jump) launch_cl_pairs<3, true>(s, p, step_off, list, st);
-    else launch_cl_pairs<3, false>(s, p, step_off, list, st);
+void launch_cluster_pairs(const DevSys& s, const Params& p, int step_off, int part, int list, cudaStream_t st, bool early) {
+    if (part != 3) launch_cl_pairs<5, true>(s, p, step_off, list, early, st);
+    else if (p.coul_jump) launch_cl_pairs<3, true>(s, p, step_off, list, early, st);
+    else launch_cl_pairs<3, false>(s, p, step_off, list, early, st);
 }
 
 void launch_cluster_collect(const DevSys& s, double* out, cudaStream_t st) {

@@ -692,10 +692,16 @@ __device__ __forceinline__ float3 bonded_grad(const Params& p, const DevSys& s, 
 // may be scheduled while its predecessor in the stream still runs.  It waits
 // here until the predecessor has completed and its writes are visible, before
 // reading anything, and then lets its own successor be scheduled.  Without a
-// programmatic predecessor the wait returns at once.
+// programmatic predecessor the wait returns at once.  So when a kernel starts,
+// every kernel of the chain before its predecessor has completed: one that
+// needs nothing of its predecessor may work first and wait last (chain_next,
+// then chain_wait, in every CTA, before it ends; its successor then has to wait
+// before it reads what the predecessor wrote).
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void chain_enter() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    chain_wait();
+    chain_next();
 }
 
 template <typename... KArgs, typename... Args>
@@ -730,7 +736,8 @@ void launch_rebuild(const DevSys& s, const Params& p, int step_off, bool force, 
 void launch_step(const DevSys& s, const Params& p, int integrator, int variant, int step_off, double hr,
                  double hout, cudaStream_t st);
 // launch_step in two parts (for per-kernel timing): the pair sums, then the step kernel.
-int launch_step_pairs(const DevSys& s, const Params& p, int integrator, int step_off, double hout, cudaStream_t st);
+int launch_step_pairs(const DevSys& s, const Params& p, int integrator, int step_off, double hr, double hout,
+                      cudaStream_t st);
 void launch_step_kernel(const DevSys& s, const Params& p, int integrator, int variant, int step_off, double hr,
                         double hout, int pre, cudaStream_t st);
 // energy: also the FP64 energy partials of the convolution (bounce_get_energies)
@@ -759,7 +766,10 @@ void launch_cluster_rebuild(const DevSys& s, const Params& p, int step_off, bool
                             bool binned = false);
 // sizes the pair kernel's resident grid once (outside any graph capture)
 void prepare_cluster_pairs();
-void launch_cluster_pairs(const DevSys& s, const Params& p, int step_off, int part, int list, cudaStream_t st);
+// early: the kernel launched before (SPME's last) makes nothing that the pair
+// sums read; they do not wait for it.
+void launch_cluster_pairs(const DevSys& s, const Params& p, int step_off, int part, int list, cudaStream_t st,
+                          bool early = false);
 void launch_cluster_collect(const DevSys& s, double* out, cudaStream_t st);
 // All-pairs tiles (tile.cu): the pair sums of `part` into the atom-indexed
 // accumulators, and their read-out (added to out[3n], accumulators cleared).
