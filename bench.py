@@ -78,7 +78,7 @@ OPS_PER_PAIR = {"f0": 66, "full": 55}
 # DRAM traffic of one launch of the F_0 pair kernel on this machine (ncu
 # dram__bytes_read.sum + dram__bytes_write.sum of k_cl_pairs<3>, the
 # BOUNCE-RESPA part of `bench.py --profile box --steps 8`; cold caches)
-PAIR_TRAFFIC = 24.08e6 + 2.6e3
+PAIR_TRAFFIC = 23.95e6 + 1.3e3
 
 
 def _peaks():

@@ -121,7 +121,7 @@ __device__ __forceinline__ double na_exact_r2(const Params& p, const double* q, 
 // Bounded by the ~35 instructions of a pair.  A warp per atom, lanes over j,
 // read 36 bytes a pair and looked its LJ parameters up in constant memory at
 // diverging addresses: 42 us for 4,500 atoms and 12 us for the sum over the
-// atoms by one CTA, where this takes 15 in all.
+// atoms by one CTA, where this takes 34 in all.
 __global__ void __launch_bounds__(NA_NT) k_na_pairs(void* scratch, int n, const double* q, const int* mol,
                                                     const __grid_constant__ Params p, unsigned lj_types, double kfix,
                                                     double* out) {

@@ -949,7 +949,8 @@ __device__ __forceinline__ void jump_lite(const DevSys& s, const Params& p, int 
 // over the SMs, are best: 12,288 atoms took 48 CTAs of eight warps, two SMs of
 // three idle.  Up to eight CTAs an SM keep every value in registers; twelve
 // fit the 98,304-atom box into one wave for a few spills around the jump
-// phases.  24.5 -> 13 us a step of 12,288 atoms, 41 -> 28 us of 98,304.
+// phases.  Alone and with cold caches 41 -> 29 us for 98,304 atoms; a step of
+// 12,288 atoms 90 -> 76 us in all.
 constexpr int LITE_T = 64, LITE_FEW = 8, LITE_MANY = 12;
 
 template <int BOUNCE, int CTAS>
