@@ -216,7 +216,7 @@ constexpr int NB_RING = 256;                   // queued clusters: < NB_QUEUE le
 
 __device__ __forceinline__ void cl_search(const DevSys& s, const Params& p, int step_off) {
     __shared__ int run_start[NB_NT], run_off[NB_NT];  // non-empty columns: first candidate, first cluster less it
-    __shared__ int wsum[NB_W];
+    __shared__ uint32_t wsum[NB_W];
     __shared__ int ring[NB_RING];
     __shared__ int bcnt[2][NB_W];
     __shared__ uint32_t acnt[2][NB_PASS * NB_W];
@@ -333,18 +333,20 @@ __device__ __forceinline__ void cl_search(const DevSys& s, const Params& p, int 
                 len = coln >= col ? max(c.col_ncl[coln] - k0, 0) : 0;
                 off = coln * c.maxcl + k0;
             }
-            // prefix over the columns: candidates (low 24 bits) and non-empty columns
-            const int v = len | (len > 0) << 24;
-            int x = v;
+            // prefix over the columns: candidates (low 24 bits) and non-empty
+            // columns (the upper 8: up to NB_NT, which a signed word does not hold)
+            static_assert(NB_NT < 256 && NB_NT * (BOUNCE_CL_MAXCOL / CL) < 1 << 24, "both counts fit their bits");
+            const uint32_t v = (uint32_t)len | (len > 0 ? 1u << 24 : 0u);
+            uint32_t x = v;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
-                const int y = __shfl_up_sync(0xffffffffu, x, o);
+                const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
                 if (lane >= o) x += y;
             }
             __syncthreads();  // (the last batch's runs are read)
             if (lane == 31) wsum[wl] = x;
             __syncthreads();
-            int total = 0;
+            uint32_t total = 0u;
 #pragma unroll
             for (int w = 0; w < NB_W; ++w) {
                 if (w == wl) x += total;
@@ -352,10 +354,10 @@ __device__ __forceinline__ void cl_search(const DevSys& s, const Params& p, int 
             }
             x -= v;
             if (len > 0) {
-                run_start[x >> 24] = x & 0xffffff;
-                run_off[x >> 24] = off - (x & 0xffffff);
+                run_start[x >> 24] = (int)(x & 0xffffffu);
+                run_off[x >> 24] = off - (int)(x & 0xffffffu);
             }
-            const int nr = total >> 24, nt = total & 0xffffff;
+            const int nr = (int)(total >> 24), nt = (int)(total & 0xffffffu);
             __syncthreads();
             int t0 = 0;
             do {  // (once where no column has a cluster, for what is left in the ring)
