@@ -27,7 +27,7 @@
 namespace {
 
 // The sub-steps of one stage: this lane's i atoms (two, packed) against the 32
-// staged j atoms.  GEN: with the index rule j > i and the minimum image.
+// staged j atoms.  GEN: with the index rule j > i (m > dj) and the minimum image.
 template <int PART, bool EW, bool CJ, bool GEN>
 __device__ __forceinline__ void tile_stage(const PairConsts& k, const float4* sh, const float4* sl, const int* sm,
                                            const float2* lj, const float2 (&h)[3], const float2 (&l)[3], float2 kq,
@@ -137,7 +137,10 @@ __global__ void __launch_bounds__(256, 2) k_tile_pairs(const __grid_constant__ D
             sh_m[wl][lane] = lane < nj ? s.mol[j0 + lane] : -1;
             __syncwarp();
             float2 gj[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-            const int dj[2] = {i[0] - j0, i[1] - j0};  // staged atom of the lane's own i atoms
+            // staged atom of the lane's own i atoms (one beyond its tile's end lies beyond every j);
+            // past the stage for an atom of a negative molecule, which takes no part: the minimum
+            // image folds its far coordinate back into a periodic box
+            const int dj[2] = {mi[0] >= 0 ? i[0] - j0 : 32, mi[1] >= 0 ? i[1] - j0 : 32};
             const bool gen = p.periodic || j0 < w.x + 32 || ((w.y >> 16) && j0 < w.x + t.tj + 32);
             if (gen)
                 tile_stage<PART, EW, CJ, true>(k, sh_h[wl], sh_l[wl], sh_m[wl], s_lj, h, l, kq, mi, ti, dj, gi, gj, np);
