@@ -75,6 +75,7 @@ struct bounce_ctx {
     cudaStream_t cap_stream = nullptr;
     cudaGraphExec_t graph[5][64] = {};  // [integrator][RESPA phase of the chunk's first step]
     long long cur_step = 0;              // host mirror of the device step counter
+    bool step_known = true;              // false from the first launch that moves the counter to the call's end (settle_step)
     bool rows_valid = false;             // rows were requested for this topology and replica layout
     bool has_pme = false;
     DevPme pme{};
@@ -912,6 +913,26 @@ int check_err(bounce_ctx* c, cudaStream_t st) {
     return BOUNCE_OK;
 }
 
+// cur_step after a call that failed on its way (a launch or the final wait
+// returned an error, for instance because the stream was being captured): how
+// far the device came only its own counter tells.
+int settle_step(bounce_ctx* c, cudaStream_t st) {
+    if (c->step_known) return BOUNCE_OK;
+    long long* at = reinterpret_cast<long long*>(c->h_out);
+    CU(cudaMemcpyAsync(at, c->d_step, sizeof(long long), cudaMemcpyDeviceToHost, st));
+    CU(cudaStreamSynchronize(st));
+    c->cur_step = *at;
+    c->step_known = true;
+    return BOUNCE_OK;
+}
+
+// The end of a call that moved the counter: cur_step holds once the device is known to have come there.
+int check_step(bounce_ctx* c, cudaStream_t st) {
+    const int r = check_err(c, st);
+    c->step_known = r != BOUNCE_ERR_CUDA;
+    return r;
+}
+
 // What happens at one step boundary: whether the reciprocal gradient is
 // evaluated there and the time hr it kicks over (see k_step).
 void plan(const bounce_ctx* c, int integ, int variant, long long step, bool& pme, double& hr, double& hout) {
@@ -1380,12 +1401,14 @@ int bounce_set_state(bounce_ctx* c, const double* q, const double* v, int64_t st
     // rows stay valid while every atom is within skin/2 of where they were
     // built (the same test as during a run); otherwise the next launch
     // rebuilds them
+    c->step_known = false;
     launch_state_in(s, c->pp, dq, dv, cur, step, c->rows_valid ? 1 : 2, st);
     c->rows_valid = true;
     c->rows_check_due = false;
     CU(cudaStreamSynchronize(st));
     c->step0 = step;
     c->cur_step = step;
+    c->step_known = true;
     c->have_state = true;
     ++c->pos_version;
     return BOUNCE_OK;
@@ -1417,13 +1440,14 @@ int bounce_get_state(bounce_ctx* c, double* q, double* v, int32_t where, void* s
 int bounce_run(bounce_ctx* c, int64_t n_steps, int32_t integ, void* stream) {
     if (!c) return BOUNCE_ERR_INVALID_ARG;
     if (!c->have_state) return fail(c, BOUNCE_ERR_STATE, "no state");
-    int r = check_run_args(c, n_steps, integ);
-    if (r) return r;
-    if (n_steps == 0) return BOUNCE_OK;
     cudaSetDevice(c->cfg.device);
     cudaStream_t st = (cudaStream_t)stream;
+    int r = settle_step(c, st);
+    if (r || (r = check_run_args(c, n_steps, integ))) return r;
+    if (n_steps == 0) return BOUNCE_OK;
     const int m = respa_period(c, integ);
     long long s0 = c->cur_step;
+    c->step_known = false;
     rows_before_run(c, integ, st);
     // head: B/2 [J] A O A at the current step
     boundary(c, integ, 0, 0, s0, st);
@@ -1445,7 +1469,7 @@ int bounce_run(bounce_ctx* c, int64_t n_steps, int32_t integ, void* stream) {
     if (integ == BOUNCE_BAOAB && c->ds.cl.on) c->rows_check_due = true;
     rows_after_run(c, integ);
     CU(cudaGetLastError());
-    return check_err(c, st);
+    return check_step(c, st);
 }
 
 int bounce_profile_steps(bounce_ctx* c, int64_t n_steps, int32_t integ, void* stream, double* kernel_ms,
@@ -1453,12 +1477,14 @@ int bounce_profile_steps(bounce_ctx* c, int64_t n_steps, int32_t integ, void* st
     if (!c) return BOUNCE_ERR_INVALID_ARG;
     if (!c->have_state) return fail(c, BOUNCE_ERR_STATE, "no state");
     if (n_steps < 1 || !kernel_ms) return fail(c, BOUNCE_ERR_INVALID_ARG, "bad profile arguments");
-    if (int r0 = check_run_args(c, n_steps, integ)) return r0;
     cudaSetDevice(c->cfg.device);
     cudaStream_t st = (cudaStream_t)stream;
+    if (int r0 = settle_step(c, st)) return r0;
+    if (int r0 = check_run_args(c, n_steps, integ)) return r0;
     std::vector<cudaEvent_t> ev(2 * (size_t)(n_steps + 1));
     for (auto& e : ev) CU(cudaEventCreate(&e));
     const long long s0 = c->cur_step;
+    c->step_known = false;
     rows_before_run(c, integ, st);
     auto timed = [&](int k, int variant, int off, long long step) {
         bool pme;
@@ -1488,7 +1514,7 @@ int bounce_profile_steps(bounce_ctx* c, int64_t n_steps, int32_t integ, void* st
     for (auto& e : ev) cudaEventDestroy(e);
     *kernel_ms = tot;
     if (launches) *launches = n_steps + 1;
-    return check_err(c, st);
+    return check_step(c, st);
 }
 
 int bounce_profile_breakdown(bounce_ctx* c, int64_t n_steps, int32_t integ, void* stream, double* ms,
@@ -1496,9 +1522,10 @@ int bounce_profile_breakdown(bounce_ctx* c, int64_t n_steps, int32_t integ, void
     if (!c) return BOUNCE_ERR_INVALID_ARG;
     if (!c->have_state) return fail(c, BOUNCE_ERR_STATE, "no state");
     if (n_steps < 1 || !ms) return fail(c, BOUNCE_ERR_INVALID_ARG, "bad profile arguments");
-    if (int r0 = check_run_args(c, n_steps, integ)) return r0;
     cudaSetDevice(c->cfg.device);
     cudaStream_t st = (cudaStream_t)stream;
+    if (int r0 = settle_step(c, st)) return r0;
+    if (int r0 = check_run_args(c, n_steps, integ)) return r0;
     constexpr int NK = 5;  // pair sums, step kernel, row rebuild, cluster rebuild, SPME
     std::vector<cudaEvent_t> ev;
     std::vector<int> kind;
@@ -1511,6 +1538,7 @@ int bounce_profile_breakdown(bounce_ctx* c, int64_t n_steps, int32_t integ, void
         return true;
     };
     const long long s0 = c->cur_step;
+    c->step_known = false;
     rows_before_run(c, integ, st);
     bool ok = true;
     auto one = [&](int variant, int off, long long step) {
@@ -1551,8 +1579,8 @@ int bounce_profile_breakdown(bounce_ctx* c, int64_t n_steps, int32_t integ, void
         if (groups) groups[kind[e]] += 1;
     }
     for (auto& e : ev) cudaEventDestroy(e);
-    if (!ok) return fail(c, BOUNCE_ERR_CUDA, "cudaEventCreate failed");
-    return check_err(c, st);
+    const int r = check_step(c, st);
+    return ok ? r : fail(c, BOUNCE_ERR_CUDA, "cudaEventCreate failed");
 }
 
 int bounce_autotune(bounce_ctx* c, int32_t integ, void* stream, bounce_tuning* out) {
@@ -1668,6 +1696,7 @@ int bounce_get_energies(bounce_ctx* c, bounce_energies* out, void* stream) {
     if (!c->have_state) return fail(c, BOUNCE_ERR_STATE, "no state");
     cudaSetDevice(c->cfg.device);
     cudaStream_t st = (cudaStream_t)stream;
+    if (int r0 = settle_step(c, st)) return r0;
     const long long step = c->cur_step;
     if (int r0 = prepare_readers(c, st)) return r0;
     launch_energies(c->ds, c->pp, (int)(step & 1), c->terms, st);
@@ -1714,6 +1743,7 @@ int bounce_pair_histogram(bounce_ctx* c, int32_t ta, int32_t tb, double r_max, i
         if (r) return r;
         c->hist_alloc = n_bins;
     }
+    if (int r0 = settle_step(c, st)) return r0;
     const long long step = c->cur_step;
     if (int r0 = prepare_readers(c, st)) return r0;
     CU(cudaMemsetAsync(c->hist, 0, n_bins * sizeof(unsigned long long), st));
@@ -1731,6 +1761,7 @@ int bounce_set_msd_reference(bounce_ctx* c, void* stream) {
         int r = dalloc(c, &c->msd_ref, 3 * (size_t)c->n);
         if (r) return r;
     }
+    if (int r0 = settle_step(c, st)) return r0;
     const long long step = c->cur_step;
     const int cur = (int)(step & 1);
     const size_t b = c->n * sizeof(double);
@@ -1747,6 +1778,7 @@ int bounce_msd(bounce_ctx* c, int32_t type, double* out, void* stream) {
     if (!c->have_msd_ref) return fail(c, BOUNCE_ERR_STATE, "no msd reference");
     cudaSetDevice(c->cfg.device);
     cudaStream_t st = (cudaStream_t)stream;
+    if (int r0 = settle_step(c, st)) return r0;
     const long long step = c->cur_step;
     launch_msd(c->ds, c->msd_ref, c->msd_ref + c->n, c->msd_ref + 2 * (size_t)c->n, (int)(step & 1), type, c->terms,
                st);
@@ -1782,6 +1814,7 @@ int bounce_compute_gradient(bounce_ctx* c, int32_t part, double* grad, int32_t w
     if (!c->have_state) return fail(c, BOUNCE_ERR_STATE, "no state");
     cudaSetDevice(c->cfg.device);
     cudaStream_t st = (cudaStream_t)stream;
+    if (int r0 = settle_step(c, st)) return r0;
     const long long step = c->cur_step;
     if (int r0 = prepare_readers(c, st)) return r0;
     const cudaMemcpyKind kind = where == BOUNCE_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
@@ -1822,6 +1855,7 @@ int bounce_jump_half(bounce_ctx* c, int64_t step, int32_t stream_id, int32_t* M,
     if (!c->have_state) return fail(c, BOUNCE_ERR_STATE, "no state");
     cudaSetDevice(c->cfg.device);
     cudaStream_t st = (cudaStream_t)stream;
+    if (int r0 = settle_step(c, st)) return r0;
     const long long cur_step = c->cur_step;
     if (c->jfilter) {
         // the stand-alone half-step draws over the full rows
@@ -1847,6 +1881,7 @@ int bounce_get_rows(bounce_ctx* c, int32_t* counts, int32_t* rows, int32_t capac
     if (!c || !counts || !rows || capacity < 1) return fail(c, BOUNCE_ERR_INVALID_ARG, "bad row arguments");
     if (!c->have_state) return fail(c, BOUNCE_ERR_STATE, "no state");
     cudaSetDevice(c->cfg.device);
+    if (int r0 = settle_step(c, nullptr)) return r0;
     if (int r0 = prepare_readers(c, nullptr)) return r0;
     CU(cudaDeviceSynchronize());
     int r = check_err(c, nullptr);
@@ -1940,6 +1975,7 @@ int bounce_pair_forward(bounce_ctx* c, const double* q, int32_t T, const double*
     if (r) return r;
     cudaSetDevice(c->cfg.device);
     cudaStream_t st = (cudaStream_t)stream;
+    if ((r = settle_step(c, st))) return r;
     const int cur = (int)(c->cur_step & 1);
     const int n = c->n;
     if (q) {
@@ -1968,6 +2004,7 @@ int bounce_pair_backward(bounce_ctx* c, int32_t T, const double* qt, const doubl
     cudaSetDevice(c->cfg.device);
     cudaStream_t st = (cudaStream_t)stream;
     if (!c->diff_part && (r = dalloc(c, &c->diff_part, diff_scratch(c->n)))) return r;
+    if ((r = settle_step(c, st))) return r;
     const int cur = (int)(c->cur_step & 1);
     const double* sums =
         launch_pair_backward(c->ds, c->pp, fq, fs, fe, T, cur, grad_forces, grad_energy, grad_pos, c->diff_part, st);
