@@ -504,11 +504,6 @@ __device__ __forceinline__ float chi_of(const Params& p, float r) {
     return s * s * s * (10.f + s * (-15.f + 6.f * s));
 }
 
-// 1: the pair sums take erfc from the CUDA library instead of 7.1.26
-#ifndef CL_LIBRARY_ERFC
-#define CL_LIBRARY_ERFC 0
-#endif
-
 // erfc(x) e^{x^2} for x >= 0 by Abramowitz and Stegun, Handbook of
 // Mathematical Functions, 7.1.26: t = 1/(1 + p x), t (a1 + t (a2 + t (a3 +
 // t (a4 + t a5)))); absolute error of erfc(x) below 1.5e-7.  The pair sums
@@ -533,11 +528,7 @@ __device__ __forceinline__ float pairsum_w(const Params& p, float r2, float qq, 
     if (p.ebeta > 0.f) {
         const float x = p.ebeta * r;
         const float e = __expf(-x * x);
-#if CL_LIBRARY_ERFC
-        wc = -qq * (erfcf(x) * ir2 + p.e2b_sqrtpi * e * ir) * ir;
-#else
         wc = -qq * (erfc_scaled_as(x) * e * ir2 + p.e2b_sqrtpi * e * ir) * ir;
-#endif
     } else {
         wc = -qq * ir2 * ir;
     }
