@@ -683,11 +683,14 @@ __device__ __forceinline__ float3 bonded_grad(const Params& p, const DevSys& s, 
 // may be scheduled while its predecessor in the stream still runs.  It waits
 // here until the predecessor has completed and its writes are visible, before
 // reading anything, and then lets its own successor be scheduled.  Without a
-// programmatic predecessor the wait returns at once.  So when a kernel starts,
-// every kernel of the chain before its predecessor has completed: one that
-// needs nothing of its predecessor may work first and wait last (chain_next,
-// then chain_wait, in every CTA, before it ends; its successor then has to wait
-// before it reads what the predecessor wrote).
+// programmatic predecessor the wait returns at once.
+// What may still run when a kernel starts: its predecessor; and, where that
+// one let it start before its own wait (chain_next first, chain_wait in every
+// CTA before it ends: the pair sums beside SPME's gather), also the kernel
+// before that, which must have waited first.  Everything earlier has
+// completed.  So before its wait a kernel may read only what neither of the two
+// writes, and write nothing that they read or write; after the wait both have
+// completed.
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void chain_enter() {

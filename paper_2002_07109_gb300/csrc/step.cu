@@ -958,10 +958,11 @@ __global__ void __launch_bounds__(LITE_T, CTAS) k_step_lite(const __grid_constan
                                                                    const __grid_constant__ Params p, int variant,
                                                                    int step_off, double hr, int ext, double hout) {
     __shared__ unsigned long long cnt[4];
-    // Where the kernel before is the pair kernel, only its sums are waited for:
-    // it began after every other kernel of the chain had ended (chain_enter),
-    // so the atoms' state and the bonded terms are read and evaluated while
-    // its last warps still work.
+    // Where the kernel before is a pair kernel, the atoms' state and the bonded
+    // terms are read and evaluated while its last warps still work.  SPME's
+    // gather may still run then too, where the pair sums began beside it: before
+    // the wait only what neither of the two writes may be read, not the sums
+    // (acc) and not the reciprocal gradient (grecip).
     const bool sums = !(ext && hout == 0.0);
     if (!sums) chain_enter();
     if (threadIdx.x < 4) cnt[threadIdx.x] = 0ull;
