@@ -1,27 +1,29 @@
 // Pair sums over clusters of atoms (the F_0 share of every pair, Sec. IV.A /
 // Sec. V, and BAOAB's full pair gradient), for systems with a finite cutoff.
 //
-// Build (four gated launches; each returns at once unless the cluster
+// Build (three gated launches; each returns at once unless the cluster
 // rebuild flag is raised -- the step kernel raises it when an atom has moved
-// more than skin/2 since the build):
-//   1. column of every atom on a grid over (x, y), counts; the CTA finishing
-//      last scans the counts;
-//   2. scatter of the atom indices into column order;
-//   3. one CTA per column sorts its atoms by (z, index) (bitonic sort in
-//      shared memory: the order, hence every cluster, is deterministic),
-//      cuts them into clusters of BOUNCE_CL and writes the slot-ordered
-//      copies of the split positions, the molecule ids, the slot of every
-//      atom and the bounding box of every cluster;
-//   4. one warp per cluster I collects the atoms of the clusters J >= I of
-//      the columns in reach that lie within the search radius of I's box
-//      (minimum image per axis), in a fixed order, with the periodic image
-//      of each; the CTA finishing last clears the flag and raises the prune
-//      flag.
-// Prune (a fifth gated launch, also raised by the step kernel when an atom
-// has moved half the prune skin since the last prune): the entries of each
-// list within r + prune skin of some atom of I at the current positions,
-// so that the pair kernel reads a list close to the pairs it must evaluate
-// while the outer lists, with a larger skin, are rebuilt rarely.
+// more than half the skin since the build):
+//   1. k_bins (nlist.cu): the atoms counted into columns of a grid over (x, y),
+//      the counts scanned, the atom indices scattered into column order; one
+//      launch, which bins the candidate rows' cells too;
+//   2. k_cl_sort: one CTA per column sorts its atoms by (z, index) (bitonic
+//      sort in shared memory: the order, hence every cluster, is
+//      deterministic), cuts them into clusters of BOUNCE_CL and writes the
+//      slot-ordered copies of the split positions, the molecule ids, the slot
+//      of every atom and the bounding box of every cluster;
+//   3. k_cl_lists: one CTA per cluster I collects the atoms of the clusters
+//      J >= I of the columns in reach that lie within the search radius of I's
+//      box (minimum image per axis), in a fixed order, with the periodic image
+//      of each.
+// Prune (in the third launch, which its own flag opens too: the step kernel
+// raises it when an atom has moved half the prune skin since the last prune):
+// the entries of each list within r + prune skin of some atom of I at the
+// current positions, so that the pair kernel reads a list close to the pairs
+// it must evaluate while the outer lists, with a larger skin, are rebuilt
+// rarely.  A CTA prunes the clusters whose lists it made itself, so that a
+// barrier of the CTA parts the two; the CTA finishing last, after every other
+// one has read the flags, clears them both.
 // Pair kernel: one warp per work item (cluster I, a chunk of its pruned
 // entries); lane = one list atom j, the 8 atoms
 // of cluster I two at a time from shared memory.  Every unordered pair inside the
