@@ -108,14 +108,19 @@ __global__ void __launch_bounds__(256, 2) k_tile_pairs(const __grid_constant__ D
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
             i[q] = w.x + q * t.tj + lane;
-            // an i atom that does not exist is placed out of reach, without charge
+            // an i atom that does not exist, or takes no part (of a negative molecule), is placed
+            // out of reach, without charge, and beyond every j: the minimum image folds its
+            // coordinate back into a periodic box
             float4 hi = make_float4(PAIR_FAR, PAIR_FAR, PAIR_FAR, 0.f), lo = make_float4(0.f, 0.f, 0.f, 0.f);
             mi[q] = -1;
             vi[q] = lane < (q ? w.y >> 16 : w.y & 0xffff);
             if (vi[q]) mi[q] = s.mol[i[q]];
-            if (mi[q] >= 0) {
+            vi[q] = mi[q] >= 0;
+            if (vi[q]) {
                 hi = s.phi[cur][i[q]];
                 lo = s.plo[cur][i[q]];
+            } else {
+                i[q] = 1 << 30;
             }
             (&h[0].x)[q] = hi.x;
             (&h[1].x)[q] = hi.y;
@@ -137,10 +142,7 @@ __global__ void __launch_bounds__(256, 2) k_tile_pairs(const __grid_constant__ D
             sh_m[wl][lane] = lane < nj ? s.mol[j0 + lane] : -1;
             __syncwarp();
             float2 gj[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-            // staged atom of the lane's own i atoms (one beyond its tile's end lies beyond every j);
-            // past the stage for an atom of a negative molecule, which takes no part: the minimum
-            // image folds its far coordinate back into a periodic box
-            const int dj[2] = {mi[0] >= 0 ? i[0] - j0 : 32, mi[1] >= 0 ? i[1] - j0 : 32};
+            const int dj[2] = {i[0] - j0, i[1] - j0};  // staged atom of the lane's own i atoms
             const bool gen = p.periodic || j0 < w.x + 32 || ((w.y >> 16) && j0 < w.x + t.tj + 32);
             if (gen)
                 tile_stage<PART, EW, CJ, true>(k, sh_h[wl], sh_l[wl], sh_m[wl], s_lj, h, l, kq, mi, ti, dj, gi, gj, np);
@@ -159,7 +161,7 @@ __global__ void __launch_bounds__(256, 2) k_tile_pairs(const __grid_constant__ D
                 fix_add(t.acc + i[q], (&gi[0].x)[q]);
                 fix_add(t.acc + n + i[q], (&gi[1].x)[q]);
                 fix_add(t.acc + 2 * n + i[q], (&gi[2].x)[q]);
-                npair += mi[q] >= 0 ? np[q] : 0;
+                npair += np[q];
             }
     }
     npair = warp_sum_i(npair);
